@@ -85,9 +85,6 @@ def measured_hbm_gbs() -> float:
 # digest of the kernel's sources at capture time: a changed kernel has no entry and reports null
 # traffic, not stale counters.  profiles/ holds the capture summaries.
 TRAFFIC = {
-    # jacobi_reg_kernel tier 0xa01, 10 000 64x64 matrices: 164.61 MB read + 277.57 MB written, per
-    # 20 000-matrix launch (profiles/jacobi_reg_qr_svd64_qr128.md)
-    "jacobi_reg:657c5a9dca399a6b": 2 * (164.607744e6 + 277.571072e6),
     # qr_warp_kernel<float, 128, 1>, 10 000 128x32 matrices: 164.79 MB read + 146.25 MB written, per
     # 20 000-matrix launch (re-captured after the CTA QR kernel's load phase changed in the same file)
     "qr:228caeb56544bd00": 2 * (164.788992e6 + 146.252800e6),
@@ -353,8 +350,9 @@ class SvdQr64:
         achieved = fl / (kernel_ms * 1e-3) / 1e12
         tier = int(self.tuned["tier"])
         reg = (tier & 0xff) == bs.TIER_REGISTER
-        kname = ("jacobi_reg_kernel" if reg else "jacobi_smem_kernel") + f" (tier {tier:#x})"
-        traffic = TRAFFIC.get("jacobi_reg:" + kernel_digest("jacobi_reg.cu")) if reg else None
+        # (32 slots of scaled rotations: the form with W and V in separate warps)
+        kname = ("jacobi_wv_kernel" if reg else "jacobi_smem_kernel") + f" (tier {tier:#x})"
+        traffic = TRAFFIC.get("jacobi_wv:" + kernel_digest("jacobi_wv.cu")) if reg else None
         if traffic is not None:
             traffic *= self.nb / 20000  # per launch: scales with the matrix count
         roof = {"kernel": kname, "bound": "alu", "achieved": achieved, "peak": PEAKS["fp32"]["tflops"], "unit": "TFLOP/s",
