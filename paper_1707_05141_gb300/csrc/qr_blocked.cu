@@ -92,6 +92,16 @@ __device__ __forceinline__ T* qb_X(unsigned char* ws, const QbLayout& L, int b)
     return reinterpret_cast<T*>(ws + L.off_X) + (size_t)b * L.strideX;
 }
 
+// CTAs per matrix of the copy kernels: column j of a matrix is copied by CTA j % gridDim.y, so that a few
+// large matrices use the whole GPU (8 matrices of 2000 x 600 copied by one CTA each took 2.5 ms of an
+// 11.2 ms blocked QR; at full bandwidth it is 15 us)
+inline dim3 qb_copy_grid(int batch, int cols)
+{
+    const int want = (2432 + batch - 1) / batch;   // about 16 CTAs of 256 threads on each of 152 SMs
+    const int y = want < cols ? want : cols;
+    return dim3((unsigned)batch, (unsigned)(y > 1 ? y : 1));
+}
+
 // setup: shapes, X = A or A^T (ld mm), the inner call's pointer and size arrays
 template <typename T>
 __global__ void __launch_bounds__(256) qb_setup_kernel(int batch, int max_mm, int max_nn, T* const* A, const int* M,
@@ -105,7 +115,7 @@ __global__ void __launch_bounds__(256) qb_setup_kernel(int batch, int max_mm, in
     const int mm = tr ? n : m, nn = tr ? m : n;
     const bool bad = m < 0 || n < 0 || mm > max_mm || nn > max_nn || lda < (m > 1 ? m : 1) ||
                      ldu < (m > 1 ? m : 1) || ldv < (n > 1 ? n : 1);
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && blockIdx.y == 0) {
         I.mm[b] = bad ? 0 : mm;
         I.nn[b] = bad ? 0 : nn;
         I.bad[b] = bad ? 1 : 0;
@@ -121,10 +131,9 @@ __global__ void __launch_bounds__(256) qb_setup_kernel(int batch, int max_mm, in
     if (bad) return;
     T* X = qb_X<T>(ws, L, b);
     const T* a = A[b];
-    for (size_t e = threadIdx.x; e < (size_t)mm * nn; e += blockDim.x) {
-        const int j = (int)(e / mm), i = (int)(e - (size_t)j * mm);
-        X[e] = tr ? a[(size_t)i * lda + j] : a[(size_t)j * lda + i];
-    }
+    for (int j = blockIdx.y; j < nn; j += gridDim.y)
+        for (int i = threadIdx.x; i < mm; i += blockDim.x)
+            X[(size_t)j * mm + i] = tr ? a[(size_t)i * lda + j] : a[(size_t)j * lda + i];
 }
 
 // panel p: factor X(j0:mm, j0:j0+32) on chip, write reflectors and R back, form T
@@ -322,10 +331,9 @@ __global__ void __launch_bounds__(256) qb_rt_kernel(unsigned char* ws, QbLayout 
     const T* X = qb_X<T>(ws, L, b);
     const T* rd = reinterpret_cast<const T*>(ws + L.off_rd) + (size_t)b * L.strideRd;
     T* Rt = reinterpret_cast<T*>(ws + L.off_Rt) + (size_t)b * L.strideRt;
-    for (size_t e = threadIdx.x; e < (size_t)nn * nn; e += blockDim.x) {
-        const int j = (int)(e / nn), i = (int)(e - (size_t)j * nn);   // Rt(i, j) = R(j, i)
-        Rt[e] = i > j ? X[(size_t)i * mm + j] : (i == j ? rd[i] : T(0));
-    }
+    for (int j = blockIdx.y; j < nn; j += gridDim.y)                     // Rt(i, j) = R(j, i)
+        for (int i = threadIdx.x; i < nn; i += blockDim.x)
+            Rt[(size_t)j * nn + i] = i > j ? X[(size_t)i * mm + j] : (i == j ? rd[i] : T(0));
 }
 
 // the left vectors [V~; 0]: rows nn .. mm-1 zeroed; bad shapes marked again (the inner call saw
@@ -361,7 +369,7 @@ __global__ void __launch_bounds__(256) qbq_setup_kernel(int max_mm, int max_nn, 
     const int ldq = Q ? LDQ[b] : 1, ldr = R ? LDR[b] : 1;
     const bool bad = m < 0 || n < 0 || m < n || m > max_mm || n > max_nn || lda < (m > 1 ? m : 1) ||
                      (Q && ldq < (m > 1 ? m : 1)) || (R && ldr < (n > 1 ? n : 1));
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && blockIdx.y == 0) {
         I.mm[b] = bad ? 0 : m;
         I.nn[b] = bad ? 0 : n;
         I.bad[b] = bad ? 1 : 0;
@@ -370,10 +378,8 @@ __global__ void __launch_bounds__(256) qbq_setup_kernel(int max_mm, int max_nn, 
     if (bad) return;
     T* X = qb_X<T>(ws, L, b);
     const T* a = A[b];
-    for (size_t e = threadIdx.x; e < (size_t)m * n; e += blockDim.x) {
-        const int j = (int)(e / m), i = (int)(e - (size_t)j * m);
-        X[e] = a[(size_t)j * lda + i];
-    }
+    for (int j = blockIdx.y; j < n; j += gridDim.y)
+        for (int i = threadIdx.x; i < m; i += blockDim.x) X[(size_t)j * m + i] = a[(size_t)j * lda + i];
 }
 
 // R (n x n: X's strict upper triangle, the diagonal from rd, exact zeros below) and Q = [I; 0]
@@ -390,18 +396,15 @@ __global__ void __launch_bounds__(256) qbq_out_kernel(T* const* Q, const int* LD
     if (R) {
         T* r = R[b];
         const int ldr = LDR[b];
-        for (size_t e = threadIdx.x; e < (size_t)nn * nn; e += blockDim.x) {
-            const int j = (int)(e / nn), i = (int)(e - (size_t)j * nn);
-            r[(size_t)j * ldr + i] = i < j ? X[(size_t)j * mm + i] : (i == j ? rd[i] : T(0));
-        }
+        for (int j = blockIdx.y; j < nn; j += gridDim.y)
+            for (int i = threadIdx.x; i < nn; i += blockDim.x)
+                r[(size_t)j * ldr + i] = i < j ? X[(size_t)j * mm + i] : (i == j ? rd[i] : T(0));
     }
     if (Q) {
         T* q = Q[b];
         const int ldq = LDQ[b];
-        for (size_t e = threadIdx.x; e < (size_t)mm * nn; e += blockDim.x) {
-            const int j = (int)(e / mm), i = (int)(e - (size_t)j * mm);
-            q[(size_t)j * ldq + i] = i == j ? T(1) : T(0);
-        }
+        for (int j = blockIdx.y; j < nn; j += gridDim.y)
+            for (int i = threadIdx.x; i < mm; i += blockDim.x) q[(size_t)j * ldq + i] = i == j ? T(1) : T(0);
     }
 }
 
@@ -573,6 +576,386 @@ __global__ void __launch_bounds__(256) qb_panel_cluster_kernel(int p, int cs, un
     cluster.sync();   // no CTA leaves while CTA 0 may still read its shared memory
 }
 
+// ---- the blocked QR's own panel and block-reflector kernels (batched_qr_blocked) ----
+//
+// The preconditioned block tier keeps the kernels above: its singular vectors of the smallest values move
+// with the last bit of R, so its factorisation stays the one it was.  The QR itself is free to sum in
+// another order, and these sum in parallel.
+
+constexpr int kQwWarps = 16;                  // warps that own two panel columns each
+constexpr int kQwThreads = 32 * (kQwWarps + 1);   // and one that forms T
+
+// Panel p of matrix blockIdx.x / cs: CTA `rank` of its cluster holds panel rows [rank * 32 RPL, ...) in
+// registers, warp w the columns 2 w and 2 w + 1 (lane: rows lane + 32 t).  One reduction per column: the
+// raw pivot x (zero above row c) is multiplied with all 32 columns at once, since with v = (x + sg alpha
+// e_c) inv the products v^T x_j (the update of column j > c) and v_j^T v (the entry of V^T V for T, j < c)
+// are inv (x^T x_j + sg alpha x_j(c)); norm, updates and T come from the same 32 sums.  They are pushed to
+// every CTA of the cluster (distributed shared memory), so a column costs one cluster barrier and one CTA
+// barrier.  Bound by that latency.  A 2000-row panel (8 matrices, 4-CTA clusters of 500 rows) took 245 us
+// with the panel in shared memory, two cluster barriers and three passes per column; it takes 53 us here.
+template <typename T, int RPL>
+__global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, unsigned char* ws, QbLayout L, QbInts I)
+{
+    __shared__ T pub[2][RPL * 32];            // the pivot column of this CTA's rows
+    __shared__ T xch[2][kClusterMax][kPw];    // the CTAs' partial products with the pivot
+    __shared__ T row[2][kPw];                 // row c of the panel
+    __shared__ T Gs[kPw][kPw + 1], Ts[kPw][kPw + 1];   // V^T V (above the diagonal) and T (row i, column c)
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
+    const int b = blockIdx.x / cs;
+    const int mm = I.mm[b], nn = I.nn[b];
+    const int j0 = p * kPw;
+    if (j0 >= nn) return;                     // the whole cluster (one matrix) leaves together
+    const int rows = mm - j0, r0 = rank * 32 * RPL;
+    const int nr = rows - r0 < 0 ? 0 : (rows - r0 > 32 * RPL ? 32 * RPL : rows - r0);
+    const int vcols = nn - j0 < kPw ? nn - j0 : kPw;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool owner = warp < kQwWarps;
+    T* X = qb_X<T>(ws, L, b) + (size_t)j0 * mm + j0 + r0;   // panel element (row r0, column 0)
+    T x[2][RPL];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int t = 0; t < RPL; ++t) {
+            const int c = 2 * warp + q, r = lane + 32 * t;
+            x[q][t] = (owner && c < vcols && r < nr) ? X[(size_t)c * mm + r] : T(0);
+        }
+    if (warp == 0) {
+#pragma unroll
+        for (int t = 0; t < RPL; ++t) pub[0][lane + 32 * t] = x[0][t];
+    }
+    for (int e = threadIdx.x; e < kPw * (kPw + 1); e += blockDim.x) (&Ts[0][0])[e] = T(0);
+    T* rd = reinterpret_cast<T*>(ws + L.off_rd) + (size_t)b * L.strideRd + j0;
+    // T's column k (lane i: row i): T(k, k) = 2, T(0:k, k) = -2 T(0:k, 0:k) G(0:k, k)
+    auto t_column = [&](int k) {
+        T s = T(0);
+        for (int e = 0; e < k; ++e) s = fma(Ts[lane][e], Gs[e][k], s);
+        if (lane <= k) Ts[lane][k] = lane == k ? T(2) : T(-2) * s;
+    };
+    if (cs > 1) cluster.sync();               // every CTA of the cluster runs before the first push
+    else __syncthreads();
+    for (int c = 0; c < vcols; ++c) {
+        const int buf = c & 1;
+        if (owner) {
+            T s[2] = {T(0), T(0)};
+#pragma unroll
+            for (int t = 0; t < RPL; ++t) {
+                const T v = pub[buf][lane + 32 * t];
+                s[0] = fma(v, x[0][t], s[0]);
+                s[1] = fma(v, x[1][t], s[1]);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+                s[1] += __shfl_xor_sync(0xffffffffu, s[1], o);
+            }
+            const T e0 = __shfl_sync(0xffffffffu, x[0][0], c), e1 = __shfl_sync(0xffffffffu, x[1][0], c);
+            if (lane < cs) {
+                T* px = &xch[buf][rank][2 * warp];
+                T* pr = &row[buf][2 * warp];
+                if (cs > 1) {
+                    px = cluster.map_shared_rank(px, lane);
+                    pr = cluster.map_shared_rank(pr, lane);
+                }
+                px[0] = s[0];
+                px[1] = s[1];
+                if (rank == 0) {
+                    pr[0] = e0;
+                    pr[1] = e1;
+                }
+            }
+        } else if (rank == 0 && c > 0) {
+            t_column(c - 1);
+            __syncwarp();
+        }
+        if (cs > 1) cluster.sync();
+        else __syncthreads();
+        if (owner) {
+            T tot = T(0), s[2] = {T(0), T(0)};
+            for (int k = 0; k < cs; ++k) {
+                tot += xch[buf][k][c];
+                s[0] += xch[buf][k][2 * warp];
+                s[1] += xch[buf][k][2 * warp + 1];
+            }
+            const T x0 = row[buf][c];
+            const T alpha = dsqrt(tot);
+            const T sa = x0 >= T(0) ? alpha : -alpha;   // sign(x0) alpha
+            const T inv = alpha > T(0) ? drsqrt(T(2) * alpha * (alpha + dabs(x0))) : T(0);
+            const T vc = (x0 + sa) * inv;               // v's entry in row c
+            T w[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int j = 2 * warp + q;
+                const T z = inv * fma(sa, row[buf][j], s[q]);
+                w[q] = j > c ? T(-2) * z : T(0);
+                if (j < c && rank == 0 && lane == 0) Gs[j][c] = z;
+            }
+            if (rank == 0 && warp == 0 && lane == 0) rd[c] = alpha > T(0) ? -sa : T(0);
+#pragma unroll
+            for (int t = 0; t < RPL; ++t) {
+                T v = pub[buf][lane + 32 * t] * inv;
+                if (t == 0 && rank == 0 && lane == c) v = vc;
+                x[0][t] = fma(w[0], v, x[0][t]);
+                x[1][t] = fma(w[1], v, x[1][t]);
+                if (c >> 1 == warp && !(t == 0 && rank == 0 && lane < c)) {   // column c becomes v
+                    if (c & 1) x[1][t] = v;
+                    else x[0][t] = v;
+                }
+            }
+            if ((c + 1) >> 1 == warp && c + 1 < vcols) {   // publish the next pivot, zero above its row
+#pragma unroll
+                for (int t = 0; t < RPL; ++t) {
+                    const T y = (c + 1) & 1 ? x[1][t] : x[0][t];
+                    pub[buf ^ 1][lane + 32 * t] = t == 0 && rank == 0 && lane <= c ? T(0) : y;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (owner) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int t = 0; t < RPL; ++t) {
+                const int c = 2 * warp + q, r = lane + 32 * t;
+                if (c < vcols && r < nr) X[(size_t)c * mm + r] = x[q][t];
+            }
+    } else if (rank == 0) {
+        t_column(vcols - 1);
+        __syncwarp();
+        T* Tg = reinterpret_cast<T*>(ws + L.off_T) + (size_t)b * L.strideT + (size_t)p * kPw * kPw;
+        for (int k = 0; k < kPw; ++k) Tg[k * kPw + lane] = Ts[lane][k];   // column-major (columns past vcols: 0)
+    }
+}
+
+// Block reflector of panel p applied to a 32-column tile of C, as qb_apply_kernel, by a cluster of cs CTAs
+// that split the rows: CTA `rank` stages slabs of SR rows of V and C in shared memory (rank, rank + cs, ...),
+// forms its share of V^T C in 4 x 4 register blocks (four groups of 64 threads over the slab's rows), the
+// cluster adds the shares through distributed shared memory, and each CTA updates its rows from the slab it
+// still holds (one read and one write of C when cs slabs cover the rows).  Bound by FMA issue and the wave
+// count: 37 applications of the 8 x 2000 x 600 case 3.3 ms with one CTA per tile streaming its rows twice
+// (2 x 2 blocks), 1.5 ms here (two CTAs per SM: 1.66; remote sums one element at a time: the same).
+template <typename T>
+struct QwDims {
+    static constexpr int VE = 16 / (int)sizeof(T);     // elements of a 16-byte vector
+    static constexpr int SR = sizeof(T) == 4 ? 256 : 128;   // rows of a slab: 74 KB of shared memory, 3 CTAs per SM
+    static constexpr int LD = SR + VE;                 // column stride: 8 consecutive columns in distinct banks
+    static constexpr int LW = kPw + VE;
+    static constexpr size_t smem = sizeof(T) * (2 * kPw * LD + 2 * kPw * LW);
+};
+
+template <typename T>
+__device__ __forceinline__ void qw_load(const T* p, T (&v)[QwDims<T>::VE])
+{
+    if constexpr (sizeof(T) == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(p);
+        v[0] = x.x;
+        v[1] = x.y;
+        v[2] = x.z;
+        v[3] = x.w;
+    } else {
+        const double2 x = *reinterpret_cast<const double2*>(p);
+        v[0] = x.x;
+        v[1] = x.y;
+    }
+}
+template <typename T>
+__device__ __forceinline__ void qw_store(T* p, const T (&v)[QwDims<T>::VE])
+{
+    if constexpr (sizeof(T) == 4)
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else
+        *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256, 3) qw_apply_kernel(int p, int trans, int tiles, int cs, unsigned char* ws,
+                                                       QbLayout L, QbInts I, T* const* Cp, const int* LDC, int c0_base)
+{
+    typedef QwDims<T> D;
+    constexpr int VE = D::VE, SR = D::SR, LD = D::LD, LW = D::LW;
+    extern __shared__ __align__(16) unsigned char qw_sm[];
+    T* Vs = reinterpret_cast<T*>(qw_sm);      // V slab, column i at i LD
+    T* Cs = Vs + kPw * LD;                    // C slab
+    T* Wp = Cs + kPw * LD;                    // this CTA's share of V^T C: (i, c) at c LW + i
+    T* Ws = Wp + kPw * LW;                    // V^T C, then op(T) V^T C: (i, c) at i LW + c
+    T* Tsm = Wp;                              // then op(T) transposed: op(T)(i, k) at k LW + i
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
+    const int b = blockIdx.x / (tiles * cs), t = (blockIdx.x / cs) % tiles;
+    const int mm = I.mm[b], nn = I.nn[b];
+    const int j0 = p * kPw;
+    const int c0 = c0_base + kPw * t;
+    if (j0 >= nn || c0 >= nn) return;         // the whole cluster leaves together
+    const int ncol = nn - c0 < kPw ? nn - c0 : kPw;
+    const int vcols = nn - j0 < kPw ? nn - j0 : kPw;
+    T* X = qb_X<T>(ws, L, b);
+    const int ldc = Cp ? LDC[b] : mm;
+    const T* V = X + (size_t)j0 * mm + j0;
+    T* C = (Cp ? Cp[b] : X) + (size_t)c0 * ldc + j0;
+    const T* Tg = reinterpret_cast<const T*>(ws + L.off_T) + (size_t)b * L.strideT + (size_t)p * kPw * kPw;
+    const int rows = mm - j0, slabs = (rows + SR - 1) / SR;
+    const int tid = threadIdx.x;
+    const bool vv = (reinterpret_cast<uintptr_t>(V) & 15) == 0 && mm % VE == 0;
+    const bool vc = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && ldc % VE == 0;
+    T tr[kPw * kPw / 256];
+#pragma unroll
+    for (int u = 0; u < kPw * kPw / 256; ++u) tr[u] = Tg[tid + 256 * u];
+    // a slab of V (zero above the reflectors' diagonal) and of C by asynchronous copies, rows past the end zero
+    auto stage = [&](int s) {
+        const int s0 = s * SR;
+        constexpr int PC = SR / VE;   // vectors per column
+        auto column = [&](T* dst, const T* src, bool vec, int left) {   // one vector; left: valid elements
+            if (vec) {
+                left = left < 0 ? 0 : (left > VE ? VE : left);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                                 (unsigned)__cvta_generic_to_shared(dst)),
+                             "l"(left > 0 ? src : X), "r"(left * (int)sizeof(T))
+                             : "memory");
+            } else {
+#pragma unroll
+                for (int k = 0; k < VE; ++k) dst[k] = k < left ? src[k] : T(0);
+            }
+        };
+#pragma unroll 4
+        for (int e = tid; e < kPw * PC; e += 256) {
+            const int c = e / PC, r = (e % PC) * VE, left = rows - (s0 + r);
+            column(Vs + c * LD + r, V + (size_t)c * mm + s0 + r, vv, c < vcols ? left : 0);
+            column(Cs + c * LD + r, C + (size_t)c * ldc + s0 + r, vc, c < ncol ? left : 0);
+        }
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+        if (s == 0) {   // R's entries of the panel's first rows
+            __syncthreads();
+            for (int e = tid; e < kPw * kPw; e += 256)
+                if (e % kPw < e / kPw) Vs[(e / kPw) * LD + e % kPw] = T(0);
+        }
+    };
+    // share of V^T C: thread (row group g, ti, tj): V columns ti + 8 a, C columns tj + 8 b
+    const int ti = tid & 7, tj = (tid >> 3) & 7, g = tid >> 6;
+    T acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[a][c] = T(0);
+    for (int s = rank; s < slabs; s += cs) {
+        __syncthreads();
+        stage(s);
+        __syncthreads();
+#pragma unroll 2
+        for (int r = g * (SR / 4); r < (g + 1) * (SR / 4); r += VE) {
+            T v[4][VE], x[4][VE];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                qw_load(Vs + (ti + 8 * a) * LD + r, v[a]);
+                qw_load(Cs + (tj + 8 * a) * LD + r, x[a]);
+            }
+#pragma unroll
+            for (int k = 0; k < VE; ++k)
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) acc[a][c] = fma(v[a][k], x[c][k], acc[a][c]);
+        }
+    }
+    // the four row groups, one after the other, into Wp
+    for (int k = 0; k < 4; ++k) {
+        if (g == k) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    T* w = Wp + (tj + 8 * c) * LW + ti + 8 * a;
+                    *w = k == 0 ? acc[a][c] : *w + acc[a][c];
+                }
+        }
+        __syncthreads();
+    }
+    if (cs > 1) cluster.sync();
+    // the sum of the cluster's shares: the CTAs' vectors in flight together
+    for (int e = tid; e < kPw * kPw / VE; e += 256) {
+        const int c = e / (kPw / VE), i = (e % (kPw / VE)) * VE;
+        T* w = Wp + c * LW + i;
+        T x[kClusterMax][VE], s[VE];
+#pragma unroll
+        for (int k = 0; k < kClusterMax; ++k)
+            if (k < cs) qw_load(cs > 1 ? cluster.map_shared_rank(w, k) : w, x[k]);
+#pragma unroll
+        for (int u = 0; u < VE; ++u) s[u] = T(0);
+#pragma unroll
+        for (int k = 0; k < kClusterMax; ++k)
+#pragma unroll
+            for (int u = 0; u < VE; ++u)
+                if (k < cs) s[u] += x[k][u];
+#pragma unroll
+        for (int u = 0; u < VE; ++u) Ws[(i + u) * LW + c] = s[u];
+    }
+    if (cs > 1) cluster.sync();   // Wp of every CTA has been read: any of them may leave
+    else __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPw * kPw / 256; ++u) {
+        const int e = tid + 256 * u, c = e / kPw, i = e - c * kPw;   // T(i, c), column-major
+        Tsm[trans ? i * LW + c : c * LW + i] = tr[u];
+    }
+    __syncthreads();
+    {
+        // Y = op(T) W, thread: row i, four columns
+        const int i = tid >> 3, c = (tid & 7) * 4;
+        T y[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll 8
+        for (int k = 0; k < kPw; ++k) {
+            const T tk = Tsm[k * LW + i];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) y[q] = fma(tk, Ws[k * LW + c + q], y[q]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) Ws[i * LW + c + q] = y[q];
+    }
+    // C -= V Y on this CTA's slabs (the last one staged is still there): thread: VE rows, NC columns
+    constexpr int RG = SR / VE;                // row groups
+    constexpr int NC = kPw * RG / 256;         // columns per thread
+    const int rg = tid % RG, cg0 = (tid / RG) * NC;
+    const int own = rank < slabs ? (slabs - 1 - rank) / cs : -1;   // the CTA's slabs: rank + cs k, k = 0 .. own
+    for (int k = own; k >= 0; --k) {
+        const int s = rank + cs * k;
+        __syncthreads();
+        if (k != own) {
+            stage(s);
+            __syncthreads();
+        }
+        const int r = rg * VE, gr = s * SR + r;
+        T o[NC][VE];
+#pragma unroll
+        for (int j = 0; j < NC; ++j) qw_load(Cs + (cg0 + j) * LD + r, o[j]);
+#pragma unroll 4
+        for (int i = 0; i < kPw; ++i) {
+            T v[VE];
+            qw_load(Vs + i * LD + r, v);
+#pragma unroll
+            for (int j = 0; j < NC; j += VE) {
+                T y[VE];
+                qw_load(Ws + i * LW + cg0 + j, y);
+#pragma unroll
+                for (int u = 0; u < VE; ++u)
+#pragma unroll
+                    for (int e = 0; e < VE; ++e) o[j + u][e] = fma(-v[e], y[u], o[j + u][e]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            if (cg0 + j >= ncol) break;
+            T* d = C + (size_t)(cg0 + j) * ldc + gr;
+            if (vc && gr + VE <= rows) {
+                qw_store(d, o[j]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < VE; ++e)
+                    if (gr + e < rows) d[e] = o[j][e];
+            }
+        }
+    }
+}
+
 }  // namespace
 
 // rows of the tallest panel one CTA factors: its 32 columns in 200 KiB of shared memory
@@ -667,7 +1050,7 @@ int launch_block_jacobi_qr(int batch, int max_m, int max_n, int bw, int method, 
     int* ip = reinterpret_cast<int*>(ws + L.off_int);
     int** slots[7] = {&I.mm, &I.nn, &I.bad, &I.ldL, &I.ldR, &I.n2, &I.ldRt};
     for (int i = 0; i < 7; ++i) *slots[i] = ip + (size_t)i * batch;
-    qb_setup_kernel<T><<<batch, 256, 0, st>>>(batch, mm, nn, (T* const*)A, M, N, LDA, (T* const*)U, LDU, (T* const*)V,
+    qb_setup_kernel<T><<<qb_copy_grid(batch, nn), 256, 0, st>>>(batch, mm, nn, (T* const*)A, M, N, LDA, (T* const*)U, LDU, (T* const*)V,
                                               LDV, ws, L, I, Pp, info);
     if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
     constexpr size_t apply_smem = qb_apply_smem<T>();
@@ -685,7 +1068,7 @@ int launch_block_jacobi_qr(int batch, int max_m, int max_n, int bw, int method, 
                                                                               nullptr, p * kPw + kPw);
         if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
     }
-    qb_rt_kernel<T><<<batch, 256, 0, st>>>(ws, L, I);
+    qb_rt_kernel<T><<<qb_copy_grid(batch, nn), 256, 0, st>>>(ws, L, I);
     if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
     // block Jacobi on R^T: its left vectors U~ are X's right vectors, its right vectors V~ go to the
     // top of X's left-vector output
@@ -712,6 +1095,57 @@ size_t qr_blocked_workspace(int batch, int max_m, int max_n)
     return qb_layout<T>(batch, max_m > 1 ? max_m : 1, max_n > 1 ? max_n : 1, 32, 0, false).total;
 }
 
+// launch with thread-block clusters of cs CTAs along x (cs 1: an ordinary launch)
+template <typename... KArgs, typename... Args>
+static int qw_launch(void (*kern)(KArgs...), int grid, int threads, size_t smem, int cs, cudaStream_t st, Args... args)
+{
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return BSVD_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cs > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...) == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
+}
+
+// panel p of matrices whose panels have at most `rows` rows: one CTA up to 512 rows (no cluster barrier),
+// else clusters of CTAs of 512 rows, beyond 8 of those taller CTAs (registers: 2 x 48 rows a lane)
+template <typename T>
+static int qw_launch_panel(int p, int batch, int rows, unsigned char* ws, const QbLayout& L, const QbInts& I,
+                           cudaStream_t st)
+{
+    int cs = (rows + 511) / 512;
+    if (cs > kClusterMax) cs = kClusterMax;
+    const int rpl = ((rows + cs - 1) / cs + 31) / 32;
+    void (*kern)(int, int, unsigned char*, QbLayout, QbInts);
+    if (rpl <= 4) kern = qw_panel_kernel<T, 4>;
+    else if (rpl <= 8) kern = qw_panel_kernel<T, 8>;
+    else if (rpl <= 16) kern = qw_panel_kernel<T, 16>;
+    else if (rpl <= 24) kern = qw_panel_kernel<T, 24>;
+    else if (sizeof(T) == 4 && rpl <= 48) kern = qw_panel_kernel<T, sizeof(T) == 4 ? 48 : 24>;
+    else return BSVD_ERR_UNSUPPORTED;
+    return qw_launch(kern, batch * cs, kQwThreads, 0, cs, st, p, cs, ws, L, I);
+}
+
+// CTAs per tile of the block reflector: enough slabs of rows to fill the GPU, at most the slabs there are
+template <typename T>
+static int qw_apply_cluster(int batch, int tiles, int rows)
+{
+    const int slabs = (rows + QwDims<T>::SR - 1) / QwDims<T>::SR;
+    int cs = 1;
+    while (cs < kClusterMax && cs < slabs && (long long)batch * tiles * cs < 456) cs *= 2;   // 3 CTAs on each of 152 SMs
+    return cs;
+}
+
 template <typename T>
 int launch_qr_blocked(int batch, int max_m, int max_n, void* const* A, const int* M, const int* N, const int* LDA,
                       void* const* Q, const int* LDQ, void* const* R, const int* LDR, int* info, void* ws_v,
@@ -725,31 +1159,27 @@ int launch_qr_blocked(int batch, int max_m, int max_n, void* const* A, const int
     int* ip = reinterpret_cast<int*>(ws + L.off_int);
     int** slots[7] = {&I.mm, &I.nn, &I.bad, &I.ldL, &I.ldR, &I.n2, &I.ldRt};
     for (int i = 0; i < 7; ++i) *slots[i] = ip + (size_t)i * batch;
-    qbq_setup_kernel<T><<<batch, 256, 0, st>>>(max_m, max_n, (T* const*)A, M, N, LDA, (T* const*)Q, LDQ, (T* const*)R,
+    qbq_setup_kernel<T><<<qb_copy_grid(batch, max_n), 256, 0, st>>>(max_m, max_n, (T* const*)A, M, N, LDA, (T* const*)Q, LDQ, (T* const*)R,
                                                LDR, ws, L, I, info);
     if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
-    constexpr size_t apply_smem = qb_apply_smem<T>();
-    if (apply_smem > 48 * 1024 &&
-        cudaFuncSetAttribute(qb_apply_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem) !=
-            cudaSuccess)
-        return BSVD_ERR_CUDA;
+    // 32-column panels, each followed by the update of the trailing columns
     const int P = (max_n + kPw - 1) / kPw;
     for (int p = 0; p < P; ++p) {
-        const int rc = qb_launch_panel<T>(p, batch, max_m, ws, L, I, st);
-        if (rc != BSVD_SUCCESS) return rc;
-        if (p + 1 < P)
-            qb_apply_kernel<T><<<batch * (P - p - 1), 256, apply_smem, st>>>(p, 1, P - p - 1, ws, L, I, nullptr,
-                                                                              nullptr, p * kPw + kPw);
-        if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
-    }
-    qbq_out_kernel<T><<<batch, 256, 0, st>>>((T* const*)Q, LDQ, (T* const*)R, LDR, ws, L, I);
-    if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
-    if (Q) {
-        for (int p = P - 1; p >= 0; --p) {
-            qb_apply_kernel<T><<<batch * (P - p), 256, apply_smem, st>>>(p, 0, P - p, ws, L, I, (T* const*)Q, LDQ,
-                                                                          p * kPw);
-            if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
+        int rc = qw_launch_panel<T>(p, batch, max_m - p * kPw, ws, L, I, st);
+        if (rc == BSVD_SUCCESS && p + 1 < P) {
+            const int tiles = P - p - 1, cs = qw_apply_cluster<T>(batch, tiles, max_m - p * kPw);
+            rc = qw_launch(qw_apply_kernel<T>, batch * tiles * cs, 256, QwDims<T>::smem, cs, st, p, 1, tiles, cs, ws, L, I,
+                           (T* const*)nullptr, (const int*)nullptr, p * kPw + kPw);
         }
+        if (rc != BSVD_SUCCESS) return rc;
+    }
+    qbq_out_kernel<T><<<qb_copy_grid(batch, max_n), 256, 0, st>>>((T* const*)Q, LDQ, (T* const*)R, LDR, ws, L, I);
+    if (cudaGetLastError() != cudaSuccess) return BSVD_ERR_CUDA;
+    for (int p = P - 1; Q && p >= 0; --p) {
+        const int tiles = P - p, cs = qw_apply_cluster<T>(batch, tiles, max_m - p * kPw);
+        const int rc = qw_launch(qw_apply_kernel<T>, batch * tiles * cs, 256, QwDims<T>::smem, cs, st, p, 0, tiles, cs,
+                                 ws, L, I, (T* const*)Q, LDQ, p * kPw);
+        if (rc != BSVD_SUCCESS) return rc;
     }
     return BSVD_SUCCESS;
 }
