@@ -1,60 +1,129 @@
-// jacobi_rx.cu -- one-sided Jacobi SVD of FP32 matrices up to 128 x 128 with the columns resident
-// in registers and the pair exchange through shared memory (Algorithm 2, Section 2.2; the
-// shared-memory kernel of Section 5, re-arranged for sm_103a).
+// jacobi_rx.cu -- one-sided Jacobi SVD of FP32 matrices up to 128 x 128, one CTA per matrix, W and the
+// accumulated rotations V in registers of different warps (Algorithm 2, Section 2.2; the shared-memory
+// kernel of Section 5, re-arranged for sm_103a).
 //
-// The shared tier (jacobi_smem.cu) keeps W and V in shared memory and streams both columns of every
-// pair through registers at every step: eight shared-memory accesses per row of a pair, which bound
-// it by shared-memory bandwidth.  Here each pair slot's G lanes keep their rows of the slot's two W
-// columns and two V columns in registers for the whole factorisation.  The pair ordering is the
-// odd-even transposition with exchange of the register tier (2 NS positions, every processed pair
-// swaps positions, 2 NS steps per sweep), so between steps exactly one column per slot moves to the
-// neighbouring slot: it is written to a double-buffered exchange area in shared memory and read back
-// by the neighbour after the step's one barrier.  A row of a pair then costs one shared store and one
-// shared load for W and the same for V, half the traffic of the shared tier, and the rotation's
-// arithmetic runs on registers.
-//
-// Layout: slot s (0 <= s < NS = np / 2) has lanes s G .. s G + G - 1; lane g holds rows g + G k of
-// its columns (k < RW for W, k < RV for V).  Even steps pair positions (2s, 2s + 1), odd steps
-// (2s + 1, 2s + 2); on odd steps the wrap slot NS - 1, holding positions 2 NS - 1 and 0, idles.
+// The pair ordering is the odd-even transposition with exchange of the register tier: 2 NS positions,
+// even steps pair (2s, 2s + 1), odd steps (2s + 1, 2s + 2), every processed pair swaps positions, 2 NS
+// steps per sweep; on odd steps the wrap slot NS - 1, holding positions 2 NS - 1 and 0, idles.
+//   W warps (8)  slot s is lanes 4 s .. 4 s + 3; lane h holds the rows 4 q + h of the slot's two columns,
+//                pairs of q packed for two-element FMAs.  A Gram entry is summed in eight chains (rows mod 8)
+//                and a tree, the order in which eight lanes per slot would sum it.  One column per slot moves
+//                to the neighbouring slot each step, through a double-buffered area in shared memory (16-byte
+//                accesses) and one barrier of the eight warps.
+//   V warps (4)  thread t holds row t of V, the columns in registers by position: a step is two rotations'
+//                worth of FMAs per pair and no exchange (the swap renames registers).  The steps' (c, s) come
+//                through a ring in shared memory; the V warps run up to two double steps behind.
+// Bound by the W warps' dependent chain of a step (dot products, parameters, rotation, exchange); the V
+// warps fill the schedulers meanwhile.  With W and V in the same lanes, eight lanes a slot, both exchanged
+// through shared memory and the parameters computed eight times over, 1000 matrices of 127 x 100 took
+// 18.6 ms; it takes 13.1 ms here.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 #include "launch.cuh"
+#include "rnmath.cuh"
 
 namespace bsvd {
 
 namespace {
 
-constexpr int kRxG = 8;  // lanes per pair slot
+constexpr int kRxRows = 128, kRxSlots = 64;
+constexpr int kRxQuarter = 36, kRxLd = 4 * kRxQuarter;  // exchange area: strides of a lane's quarter column and of a
+                                                        // slot: eight lanes' 16-byte accesses in distinct banks
+constexpr int kRxWThreads = 256, kRxThreads = kRxWThreads + 128;
+constexpr unsigned kRxFull = 0xffffffffu;
 
-template <int RW>
-struct RxDims {
-    static constexpr int ldx = RW * kRxG + 8;  // exchange row stride: slots 8 banks apart
+struct RxShared {
+    float x[2][kRxSlots * kRxLd];       // columns on the move, by step parity and sending slot
+    float4 ring[2][2][kRxSlots / 2];    // per double step and step: (c, s) of two pairs
+    float sig[kRxRows];                 // singular values by column
+    int rank[kRxRows];                  // by position (-1: padding)
+    int count[8];                       // rotations of a sweep, per W warp
+    int more[2];                        // another sweep follows (by sweep parity)
 };
+
+// named barriers (0 is the CTA's): the W warps' own; ring slots full and empty, a sweep's end
+template <int ID, int N>
+__device__ __forceinline__ void rx_wait() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
+template <int ID, int N>
+__device__ __forceinline__ void rx_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
+constexpr int kRxW = 1, kRxFullBar = 2, kRxEmptyBar = 4, kRxSweep = 6;
+__device__ __forceinline__ void rx_wait_full(int slot) { slot ? rx_wait<kRxFullBar + 1, kRxThreads>() : rx_wait<kRxFullBar, kRxThreads>(); }
+__device__ __forceinline__ void rx_wait_empty(int slot) { slot ? rx_wait<kRxEmptyBar + 1, kRxThreads>() : rx_wait<kRxEmptyBar, kRxThreads>(); }
+__device__ __forceinline__ void rx_arrive_full(int slot) { slot ? rx_arrive<kRxFullBar + 1, kRxThreads>() : rx_arrive<kRxFullBar, kRxThreads>(); }
+__device__ __forceinline__ void rx_arrive_empty(int slot) { slot ? rx_arrive<kRxEmptyBar + 1, kRxThreads>() : rx_arrive<kRxEmptyBar, kRxThreads>(); }
+
+__device__ __forceinline__ float2 rx_both(float x) { return make_float2(x, x); }
+
+// this lane's two chains of x . y, added as eight lanes' butterfly over 4 would; then the butterflies over 2 and 1
+__device__ __forceinline__ float rx_dot(const float2 (&x)[16], const float2 (&y)[16])
+{
+    float2 a = rx_both(0.f);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) a = __ffma2_rn(x[q], y[q], a);
+    float s = a.x + a.y;
+    s += __shfl_xor_sync(kRxFull, s, 2);
+    s += __shfl_xor_sync(kRxFull, s, 1);
+    return s;
+}
+
+__device__ __noinline__ bool rx_rotation_slow(float al, float be, float ga, float tol, float* cs)
+{
+    return jacobi_rotation<float>(al, be, ga, tol, cs[0], cs[1]);
+}
+
+// rot(G) of jacobi_rotation<float>, the same numbers: by branch-free correctly rounded operations when every
+// lane of the warp is inside their range, else by jacobi_rotation itself
+template <typename P>
+__device__ __forceinline__ bool rx_rotation(float al, float be, float ga, P tol, float& c, float& s)
+{
+    c = 1.f;
+    s = 0.f;
+    if constexpr (sizeof(P) == 8) {
+        P cp, sp;
+        if (!jacobi_rotation<P>(P(al), P(be), P(ga), tol, cp, sp)) return false;
+        c = float(cp);
+        s = float(sp);
+        return true;
+    } else {
+        const bool pos = al > 0.f && be > 0.f;
+        const float d = be - al, g2 = 2.f * ga;
+        const bool rot = pos && !(fabsf(ga) <= tol * rn_sqrt(al) * rn_sqrt(be));
+        const float zeta = rn_div(d, g2), az = fabsf(zeta);
+        float t = rn_rcp(az + rn_sqrt(fmaf(zeta, zeta, 1.f)));
+        t = zeta >= 0.f ? t : -t;
+        const float cf = rn_rsqrt12(fmaf(t, t, 1.f));
+        auto in = [](float x) { return x >= 0x1p-100f && x <= 0x1p100f; };
+        // (the test itself needs the norms' range, the parameters the rest)
+        const bool safe = in(al) && in(be) && (!rot || (in(fabsf(g2)) && (d == 0.f || in(fabsf(d))) && az < 0x1p59f));
+        if (__any_sync(kRxFull, pos && !safe)) {
+            float cs[2];
+            if (!rx_rotation_slow(al, be, ga, tol, cs)) return false;
+            c = cs[0];
+            s = cs[1];
+            return true;
+        }
+        if (rot) {
+            c = cf;
+            s = cf * t;
+        }
+        return rot;
+    }
+}
 
 }  // namespace
 
-// P: precision of the rotation parameters and the rotation test (T, or double for FP32 data)
-template <typename T, typename P, int RW, int RV>
-__global__ void __launch_bounds__(64 * kRxG, 1)
-    jacobi_rx_kernel(int batch, int max_mm, int max_np, T* const* A, const int* M, const int* N, const int* LDA,
-                     T* const* Sout, T* const* U, const int* LDU, T* const* V, const int* LDV, double tol_in,
-                     int max_sweeps, int* info, long long* rot_out, ItemList wl)
+// P: precision of the rotation parameters and the rotation test (float, or double)
+template <typename P>
+__global__ void __launch_bounds__(kRxThreads, 1)
+    jacobi_rx_kernel(int batch, int max_mm, int max_np, float* const* A, const int* M, const int* N, const int* LDA,
+                     float* const* Sout, float* const* U, const int* LDU, float* const* V, const int* LDV,
+                     double tol_in, int max_sweeps, int* info, long long* rot_out, ItemList wl)
 {
-    constexpr int G = kRxG;
-    constexpr int LDW = RxDims<RW>::ldx;   // exchange stride, W rows
-    constexpr int LDV_ = RxDims<RV>::ldx;  // exchange stride, V rows
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nslot_max = max_np / 2;
-    T* xw = reinterpret_cast<T*>(smem_raw);               // [2][nslot_max][LDW]
-    T* xv = xw + (size_t)2 * nslot_max * LDW;             // [2][nslot_max][LDV_]
-    int* xc = reinterpret_cast<int*>(xv + (size_t)2 * nslot_max * LDV_);  // [2][nslot_max] column ids
-    T* sig = reinterpret_cast<T*>(xc + 2 * nslot_max);   // [max_np] singular values by column id
-    int* rank = reinterpret_cast<int*>(sig + max_np);     // [max_np]
-
-    const int tid = threadIdx.x;
-    const int s = tid / G;  // slot
-    const int g = tid % G;  // lane in the slot
+    RxShared& sh = *reinterpret_cast<RxShared*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool is_v = tid >= kRxWThreads;
 
     for (int b = item_first(wl, batch); b >= 0; b = item_next(wl, batch, b)) {
         const int m = M[b], n = N[b], lda = LDA[b];
@@ -65,7 +134,7 @@ __global__ void __launch_bounds__(64 * kRxG, 1)
         const int ns = np / 2;      // slots of this matrix
         const bool wantU = U != nullptr, wantV = V != nullptr;
         const int ldu = wantU ? LDU[b] : 1, ldvo = wantV ? LDV[b] : 1;
-        const bool bad = m < 0 || n < 0 || mm > max_mm || np > max_np || mm > RW * G || np > RV * G ||
+        const bool bad = m < 0 || n < 0 || mm > max_mm || np > max_np || mm > kRxRows || np > kRxRows ||
                          lda < (m > 1 ? m : 1) || (wantU && ldu < (m > 1 ? m : 1)) ||
                          (wantV && ldvo < (n > 1 ? n : 1));
         if (bad) {
@@ -80,247 +149,262 @@ __global__ void __launch_bounds__(64 * kRxG, 1)
             continue;
         }
         const bool accV = tr ? wantU : wantV;
-        const bool live = s < ns;
+        float* uw = tr ? (wantV ? V[b] : nullptr) : (wantU ? U[b] : nullptr);  // receives W / sigma
+        const int lduw = tr ? ldvo : ldu;
+        float* vw = tr ? (wantU ? U[b] : nullptr) : (wantV ? V[b] : nullptr);  // receives V
+        const int ldvw = tr ? ldu : ldvo;
 
-        // ---- W (A, or A^T) and V = I into registers; the padding column is zero ----
-        T wl_[RW], wr_[RW], vl_[RV], vr_[RV];
-        int colL = 2 * s, colR = 2 * s + 1;
-        const T* a = A[b];
+        if (!is_v) {
+            // ================================ W ================================
+            const int s = tid >> 2, h = tid & 3;
+            const bool live = s < ns, wrap = s == ns - 1;
+            const bool wrap_warp = (ns - 1) >> 3 == warp;
+            const float* a = A[b];
+            float2 L[16], R[16];   // element q: rows 8 q + h and 8 q + 4 + h
+            {
+                auto elem = [&](int c, int r) -> float {
+                    if (!live || c >= nn || r >= mm) return 0.f;
+                    return tr ? a[(size_t)r * lda + c] : a[(size_t)c * lda + r];
+                };
 #pragma unroll
-        for (int k = 0; k < RW; ++k) {
-            const int r = g + G * k;
-            T x = T(0), y = T(0);
-            if (live && r < mm) {
-                if (!tr) {
-                    if (colL < nn) x = a[(size_t)colL * lda + r];
-                    if (colR < nn) y = a[(size_t)colR * lda + r];
-                } else {
-                    if (colL < nn) x = a[(size_t)r * lda + colL];
-                    if (colR < nn) y = a[(size_t)r * lda + colR];
+                for (int q = 0; q < 16; ++q) {
+                    const int r = 8 * q + h;
+                    L[q] = make_float2(elem(2 * s, r), elem(2 * s, r + 4));
+                    R[q] = make_float2(elem(2 * s + 1, r), elem(2 * s + 1, r + 4));
                 }
             }
-            wl_[k] = x;
-            wr_[k] = y;
-        }
-#pragma unroll
-        for (int k = 0; k < RV; ++k) {
-            const int r = g + G * k;
-            vl_[k] = (r == colL) ? T(1) : T(0);
-            vr_[k] = (r == colR) ? T(1) : T(0);
-        }
+            const P tol = tol_in > 0.0 ? P(tol_in) : P(dsqrt(double(mm)) * Unit<float>::value);
+            const int sweeps_cap = max_sweeps > 0 ? max_sweeps : 30;
+            int sweep = 0, slot = 0;
+            bool converged = false;
+            long long total_rot = 0, sent = 0;
+            float4* out = reinterpret_cast<float4*>(sh.x[0] + s * kRxLd + h * kRxQuarter);
+            // (slots past NS exchange zeros with themselves)
+            const int up = !live ? s : (wrap ? 0 : s + 1), down = !live ? s : (s == 0 ? ns - 1 : s - 1);
+            const float4* from_up = reinterpret_cast<const float4*>(sh.x[0] + up * kRxLd + h * kRxQuarter);
+            const float4* from_dn = reinterpret_cast<const float4*>(sh.x[1] + down * kRxLd + h * kRxQuarter);
+            float4* out1 = reinterpret_cast<float4*>(sh.x[1] + s * kRxLd + h * kRxQuarter);
+            float2* ring = reinterpret_cast<float2*>(sh.ring);
 
-        const P tol = tol_in > 0.0 ? P(tol_in) : P(dsqrt(double(mm)) * Unit<T>::value);
-        const int sweeps_cap = max_sweeps > 0 ? max_sweeps : 30;
-        int sweep = 0;
-        bool converged = false;
-        long long total_rot = 0;
-        int par = 0;  // exchange buffer of this step
-
-        while (sweep < sweeps_cap) {
-            int rot_sweep = 0;
-            for (int st = 0; st < 2 * ns; ++st) {
-                const bool odd = st & 1;
-                const bool wrap = s == ns - 1;
-                // Gram entries of the slot's pair over this lane's rows, then over the slot's lanes
-                T al = T(0), be = T(0), ga = T(0);
+            while (sweep < sweeps_cap) {
+                int rot_sweep = 0;
+#pragma unroll 1
+                for (int it = 0; it < ns; ++it) {
+                    if (accV && sent >= 2) rx_wait_empty(slot);
+                    // even step: positions 2s and 2s + 1; the right column moves one slot down
+                    {
+                        const float al = rx_dot(L, L), be = rx_dot(R, R), ga = rx_dot(L, R);
+                        float c, sn;
+                        const bool rot = rx_rotation<P>(live ? al : 0.f, be, ga, tol, c, sn);
+                        const unsigned rots = __ballot_sync(kRxFull, rot && h == 0);
+                        rot_sweep += __popc(rots);
+                        if (accV && h == 0) ring[(2 * slot) * kRxSlots + s] = make_float2(c, sn);
+                        const float2 c2 = rx_both(c), s2 = rx_both(sn), m2 = rx_both(-sn);
+                        if (rots) {
 #pragma unroll
-                for (int k = 0; k < RW; ++k) {
-                    al = fma(wl_[k], wl_[k], al);
-                    be = fma(wr_[k], wr_[k], be);
-                    ga = fma(wl_[k], wr_[k], ga);
-                }
-                al = group_sum<G>(al);
-                be = group_sum<G>(be);
-                ga = group_sum<G>(ga);
-                P c, sn;
-                const bool rotated = live && !(odd && wrap) && jacobi_rotation<P>(P(al), P(be), P(ga), tol, c, sn);
-                if (rotated) {
-                    const T ct = T(c), st_ = T(sn);
+                            for (int q = 0; q < 16; ++q) {
+                                const float2 y = __ffma2_rn(s2, L[q], __fmul2_rn(c2, R[q]));
+                                L[q] = __ffma2_rn(c2, L[q], __fmul2_rn(m2, R[q]));
+                                R[q] = y;
+                            }
+                        }
 #pragma unroll
-                    for (int k = 0; k < RW; ++k) {
-                        const T x = wl_[k], y = wr_[k];
-                        wl_[k] = ct * x - st_ * y;
-                        wr_[k] = st_ * x + ct * y;
+                        for (int q = 0; q < 16; q += 2) out[q / 2] = make_float4(R[q].x, R[q].y, R[q + 1].x, R[q + 1].y);
+                        rx_wait<kRxW, kRxWThreads>();
+#pragma unroll
+                        for (int q = 0; q < 16; q += 2) {
+                            const float4 v = from_up[q / 2];
+                            R[q] = make_float2(v.x, v.y);
+                            R[q + 1] = make_float2(v.z, v.w);
+                        }
+                    }
+                    // odd step: positions 2s + 1 and 2s + 2; the left column moves one slot up.  The wrap slot
+                    // does not rotate: it hands over its right column and keeps its left one as the right
+                    {
+                        const float al = rx_dot(L, L), be = rx_dot(R, R), ga = rx_dot(L, R);
+                        float c, sn;
+                        const bool rot = rx_rotation<P>(live && !wrap ? al : 0.f, be, ga, tol, c, sn);
+                        const unsigned rots = __ballot_sync(kRxFull, rot && h == 0);
+                        rot_sweep += __popc(rots);
+                        // (0, 1) keeps position 2 NS - 1 apart from the zero columns past it in V
+                        if (accV && h == 0) ring[(2 * slot + 1) * kRxSlots + s] = wrap ? make_float2(0.f, 1.f) : make_float2(c, sn);
+                        const float2 c2 = rx_both(c), s2 = rx_both(sn), m2 = rx_both(-sn);
+                        if (rots) {
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) {
+                                const float2 x = __ffma2_rn(c2, L[q], __fmul2_rn(m2, R[q]));
+                                R[q] = __ffma2_rn(s2, L[q], __fmul2_rn(c2, R[q]));
+                                L[q] = x;
+                            }
+                        }
+                        if (wrap_warp) {
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) {
+                                const float2 l = L[q], r = R[q];
+                                L[q] = make_float2(wrap ? r.x : l.x, wrap ? r.y : l.y);
+                                R[q] = make_float2(wrap ? l.x : r.x, wrap ? l.y : r.y);
+                            }
+                        }
+#pragma unroll
+                        for (int q = 0; q < 16; q += 2) out1[q / 2] = make_float4(L[q].x, L[q].y, L[q + 1].x, L[q + 1].y);
+                        rx_wait<kRxW, kRxWThreads>();
+#pragma unroll
+                        for (int q = 0; q < 16; q += 2) {
+                            const float4 v = from_dn[q / 2];
+                            L[q] = make_float2(v.x, v.y);
+                            L[q + 1] = make_float2(v.z, v.w);
+                        }
                     }
                     if (accV) {
-#pragma unroll
-                        for (int k = 0; k < RV; ++k) {
-                            const T x = vl_[k], y = vr_[k];
-                            vl_[k] = ct * x - st_ * y;
-                            vr_[k] = st_ * x + ct * y;
-                        }
+                        rx_arrive_full(slot);
+                        slot ^= 1;
+                        ++sent;
                     }
                 }
-                // exchange, first half: the column that leaves the slot goes to the exchange area
-                T* ow = xw + ((size_t)par * nslot_max + s) * LDW;
-                T* ov = xv + ((size_t)par * nslot_max + s) * LDV_;
-                if (live) {
-                    // even -> odd: the right column moves one slot down; odd -> even: the left column
-                    // moves one slot up, except the wrap slot's right column (it did not rotate)
-                    const bool send_right = !odd || wrap;
-                    if (send_right) {
+                if (lane == 0) sh.count[warp] = rot_sweep;
+                rx_wait<kRxW, kRxWThreads>();
+                rot_sweep = 0;
 #pragma unroll
-                        for (int k = 0; k < RW; ++k) ow[g + G * k] = wr_[k];
-                        if (accV) {
-#pragma unroll
-                            for (int k = 0; k < RV; ++k) ov[g + G * k] = vr_[k];
-                        }
-                        if (g == 0) xc[par * nslot_max + s] = colR;
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < RW; ++k) ow[g + G * k] = wl_[k];
-                        if (accV) {
-#pragma unroll
-                            for (int k = 0; k < RV; ++k) ov[g + G * k] = vl_[k];
-                        }
-                        if (g == 0) xc[par * nslot_max + s] = colL;
-                    }
+                for (int w = 0; w < kRxWThreads / 32; ++w) rot_sweep += sh.count[w];
+                ++sweep;
+                total_rot += rot_sweep;
+                converged = rot_sweep == 0;
+                if (accV) {   // (a sweep of few columns has fewer double steps than the ring: both sides wait)
+                    if (tid == 0) sh.more[sweep & 1] = !converged && sweep < sweeps_cap;
+                    rx_wait<kRxSweep, kRxThreads>();
                 }
-                rot_sweep += __syncthreads_count(rotated && g == 0);
-                // second half: the neighbour's column comes in
-                if (live) {
-                    if (!odd) {
-                        const int src = s + 1 == ns ? 0 : s + 1;
-                        const T* iw = xw + ((size_t)par * nslot_max + src) * LDW;
-                        const T* iv = xv + ((size_t)par * nslot_max + src) * LDV_;
+                if (converged) break;
+                rx_wait<kRxW, kRxWThreads>();   // the counts have been read
+            }
+            // the last double steps' "empty" arrivals
+            if (sent >= 2) rx_wait_empty(slot);
+            if (sent >= 1) rx_wait_empty(slot ^ 1);
+
+            // ---- sigma_j = ||w_j||; position p holds column p after an even number of sweeps, 2 NS - 1 - p
+            // after an odd one (every sweep reverses the order) ----
+            const int colL = sweep & 1 ? np - 1 - 2 * s : 2 * s, colR = sweep & 1 ? colL - 1 : colL + 1;
+            const float sl = rx_dot(L, L), sr = rx_dot(R, R);
+            const float sgL = dsqrt(sl), sgR = dsqrt(sr);
+            if (live && h == 0) {
+                if (colL < nn) sh.sig[colL] = sgL;
+                if (colR < nn) sh.sig[colR] = sgR;
+            }
+            rx_wait<kRxW, kRxWThreads>();
+            // ---- descending rank, ties in column order ----
+            int rkL = 0, rkR = 0;
+            for (int j = 0; j < nn; ++j) {
+                const float sj = sh.sig[j];
+                rkL += (sj > sgL) || (sj == sgL && j < colL);
+                rkR += (sj > sgR) || (sj == sgR && j < colR);
+            }
+            if (!live || colL >= nn) rkL = -1;
+            if (!live || colR >= nn) rkR = -1;
+            if (live && h == 0) {
+                sh.rank[2 * s] = rkL;
+                sh.rank[2 * s + 1] = rkR;
+                float* s_out = Sout[b];
+                if (rkL >= 0) s_out[rkL] = sgL;
+                if (rkR >= 0) s_out[rkR] = sgR;
+            }
+            if (tid == 0) {
+                bool finite = true;
+                for (int j = 0; j < nn; ++j) finite = finite && isfinite(sh.sig[j]);
+                info[b] = !finite ? BSVD_INFO_NONFINITE : (converged ? sweep : BSVD_INFO_NOT_CONVERGED + sweep);
+                if (rot_out) rot_out[b] = total_rot;
+            }
+            __syncthreads();   // the ranks are there
+            if (uw) {
+                auto put = [&](const float2(&x)[16], int rk, float sg) {
+                    if (rk < 0) return;
+                    const float inv = sg > 0.f ? 1.f / sg : 0.f;
+                    float* col = uw + (size_t)rk * lduw;
 #pragma unroll
-                        for (int k = 0; k < RW; ++k) wr_[k] = iw[g + G * k];
-                        if (accV) {
+                    for (int q = 0; q < 16; ++q) {
+                        const int r = 8 * q + h;
+                        if (r < mm) col[r] = x[q].x * inv;
+                        if (r + 4 < mm) col[r + 4] = x[q].y * inv;
+                    }
+                };
+                put(L, rkL, sgL);
+                put(R, rkR, sgR);
+            }
+        } else {
+            // ================================ V ================================
+            const int row = tid - kRxWThreads;
+            float v[2 * kRxSlots];   // row `row` of the column at each position
+            if (accV) {
 #pragma unroll
-                            for (int k = 0; k < RV; ++k) vr_[k] = iv[g + G * k];
-                        }
-                        colR = xc[par * nslot_max + src];
-                    } else {
-                        const int src = s == 0 ? ns - 1 : s - 1;
-                        const T* iw = xw + ((size_t)par * nslot_max + src) * LDW;
-                        const T* iv = xv + ((size_t)par * nslot_max + src) * LDV_;
-                        if (wrap) {  // the wrap slot keeps its left column as the right one
+                for (int p = 0; p < 2 * kRxSlots; ++p) v[p] = p == row ? 1.f : 0.f;
+                int slot = 0, sweep = 0;
+                bool more = true;
+                while (more) {
+#pragma unroll 1
+                    for (int it = 0; it < ns; ++it) {
+                        // a double step in one pass: the odd step's pair (2p - 1, 2p) follows the even step's
+                        // pair (2p, 2p + 1), so every result goes to a register whose old value has been used
+                        rx_wait_full(slot);
+                        const float4* re = sh.ring[slot][0];
+                        const float4* ro = sh.ring[slot][1];
+                        float up = 0.f, oc = 1.f, os = 0.f;   // position 2p - 1 between the steps; its (c, s)
 #pragma unroll
-                            for (int k = 0; k < RW; ++k) wr_[k] = wl_[k];
-                            if (accV) {
+                        for (int p = 0; p < kRxSlots; p += 2) {
+                            const float4 e = re[p / 2], o = ro[p / 2];
 #pragma unroll
-                                for (int k = 0; k < RV; ++k) vr_[k] = vl_[k];
+                            for (int k = 0; k < 2; ++k) {
+                                const float c = k ? e.z : e.x, sn = k ? e.w : e.y;
+                                const float x = v[2 * (p + k)], y = v[2 * (p + k) + 1];
+                                const float lo = fmaf(sn, x, c * y), hi = fmaf(c, x, -sn * y);   // R', L'
+                                if (p + k == 0) {
+                                    v[0] = lo;
+                                } else {
+                                    v[2 * (p + k) - 1] = fmaf(os, up, oc * lo);
+                                    v[2 * (p + k)] = fmaf(oc, up, -os * lo);
+                                }
+                                up = hi;
+                                oc = k ? o.z : o.x;
+                                os = k ? o.w : o.y;
                             }
-                            colR = colL;
                         }
-#pragma unroll
-                        for (int k = 0; k < RW; ++k) wl_[k] = iw[g + G * k];
-                        if (accV) {
-#pragma unroll
-                            for (int k = 0; k < RV; ++k) vl_[k] = iv[g + G * k];
-                        }
-                        colL = xc[par * nslot_max + src];
+                        v[2 * kRxSlots - 1] = up;
+                        rx_arrive_empty(slot);
+                        slot ^= 1;
                     }
+                    rx_wait<kRxSweep, kRxThreads>();
+                    ++sweep;
+                    more = sh.more[sweep & 1] != 0;
                 }
-                par ^= 1;
             }
-            ++sweep;
-            total_rot += rot_sweep;
-            if (rot_sweep == 0) {
-                converged = true;
-                break;
-            }
-        }
-
-        // ---- sigma_j = ||w_j||, by column id ----
-        {
-            T sl = T(0), sr = T(0);
+            __syncthreads();   // the ranks are there
+            if (accV && row < nn) {
 #pragma unroll
-            for (int k = 0; k < RW; ++k) {
-                sl = fma(wl_[k], wl_[k], sl);
-                sr = fma(wr_[k], wr_[k], sr);
-            }
-            sl = group_sum<G>(sl);
-            sr = group_sum<G>(sr);
-            if (live && g == 0) {
-                if (colL < nn) sig[colL] = dsqrt(sl);
-                if (colR < nn) sig[colR] = dsqrt(sr);
-            }
-        }
-        __syncthreads();
-        // ---- descending rank, ties in column order ----
-        for (int j = tid; j < nn; j += blockDim.x) {
-            const T sj = sig[j];
-            int r = 0;
-            for (int i = 0; i < nn; ++i) {
-                const T si = sig[i];
-                r += (si > sj) || (si == sj && i < j);
-            }
-            rank[j] = r;
-        }
-        __syncthreads();
-
-        // ---- outputs from the registers: S; left vectors W / sigma; right vectors V (swapped when
-        // the working matrix is A^T) ----
-        T* s_out = Sout[b];
-        for (int j = tid; j < nn; j += blockDim.x) s_out[rank[j]] = sig[j];
-        T* uw = tr ? (wantV ? V[b] : nullptr) : (wantU ? U[b] : nullptr);  // receives W / sigma
-        const int lduw = tr ? ldvo : ldu;
-        T* vw = tr ? (wantU ? U[b] : nullptr) : (wantV ? V[b] : nullptr);  // receives V
-        const int ldvw = tr ? ldu : ldvo;
-        if (live) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int col = h ? colR : colL;
-                if (col >= nn) continue;
-                const int rk = rank[col];
-                const T sj = sig[col];
-                const T inv = sj > T(0) ? T(1) / sj : T(0);
-                if (uw) {
-#pragma unroll
-                    for (int k = 0; k < RW; ++k) {
-                        const int r = g + G * k;
-                        if (r < mm) uw[(size_t)rk * lduw + r] = (h ? wr_[k] : wl_[k]) * inv;
-                    }
-                }
-                if (vw) {
-#pragma unroll
-                    for (int k = 0; k < RV; ++k) {
-                        const int r = g + G * k;
-                        if (r < nn) vw[(size_t)rk * ldvw + r] = h ? vr_[k] : vl_[k];
-                    }
+                for (int p = 0; p < 2 * kRxSlots; ++p) {
+                    const int rk = p < np ? sh.rank[p] : -1;
+                    if (rk >= 0) vw[(size_t)rk * ldvw + row] = v[p];
                 }
             }
         }
-        if (tid == 0) {
-            bool finite = true;
-            for (int i = 0; i < nn; ++i) finite = finite && isfinite(sig[i]);
-            info[b] = !finite ? BSVD_INFO_NONFINITE : (converged ? sweep : BSVD_INFO_NOT_CONVERGED + sweep);
-            if (rot_out) rot_out[b] = total_rot;
-        }
-        __syncthreads();
+        __syncthreads();   // the shared areas are reused by the next item
     }
 }
 
-// shared memory of a launch: two exchange buffers for W and V rows, column ids, sigma and ranks
-template <typename T, int RW, int RV>
-static size_t jacobi_rx_bytes(int max_np)
-{
-    const int ns = max_np / 2;
-    return ((size_t)2 * ns * RxDims<RW>::ldx + (size_t)2 * ns * RxDims<RV>::ldx) * sizeof(T) +
-           (size_t)2 * ns * sizeof(int) + (size_t)max_np * (sizeof(T) + sizeof(int)) + 16;
-}
-
-template <typename T, typename P, int RW, int RV>
+template <typename P>
 static int launch_rx(int batch, int max_mm, int max_np, void* const* A, const int* M, const int* N, const int* LDA,
                      void* const* S, void* const* U, const int* LDU, void* const* V, const int* LDV, double tol,
                      int max_sweeps, int* info, long long* rot, cudaStream_t st, ItemList wl)
 {
-    auto kern = jacobi_rx_kernel<T, P, RW, RV>;
-    const size_t smem = jacobi_rx_bytes<T, RW, RV>(max_np);
+    auto kern = jacobi_rx_kernel<P>;
+    const size_t smem = sizeof(RxShared);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return BSVD_ERR_CUDA;
-    const int threads = (max_np / 2) * kRxG < 32 ? 32 : (max_np / 2) * kRxG;
-    const int grid = item_grid(kern, threads, smem, wl, batch, st);
+    const int grid = item_grid(kern, kRxThreads, smem, wl, batch, st);
     if (grid == 0) return BSVD_ERR_CUDA;
-    kern<<<grid, threads, smem, st>>>(batch, max_mm, max_np, (T* const*)A, M, N, LDA, (T* const*)S, (T* const*)U, LDU,
-                                      (T* const*)V, LDV, tol, max_sweeps, info, rot, wl);
+    kern<<<grid, kRxThreads, smem, st>>>(batch, max_mm, max_np, (float* const*)A, M, N, LDA, (float* const*)S,
+                                  (float* const*)U, LDU, (float* const*)V, LDV, tol, max_sweeps, info, rot, wl);
     return cudaGetLastError() == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
 }
 
-// FP32 matrices with max(m, n) <= 128 (16 rows of W and of V per lane; more rows would exceed the
-// 128 registers a thread has at 512 threads).  Returns BSVD_ERR_UNSUPPORTED for other shapes (the
-// caller then takes the shared tier).
+// FP32 matrices with max(m, n) <= 128.  Returns BSVD_ERR_UNSUPPORTED for other shapes (the caller then takes
+// the shared tier).
 int launch_jacobi_rx(int batch, int max_m, int max_n, void* const* A, const int* M, const int* N, const int* LDA,
                      void* const* S, void* const* U, const int* LDU, void* const* V, const int* LDV, double tol,
                      int max_sweeps, int* info, long long* rot, cudaStream_t st, ItemList wl, bool p64)
@@ -328,11 +412,11 @@ int launch_jacobi_rx(int batch, int max_m, int max_n, void* const* A, const int*
     const int max_mm = max_m > max_n ? max_m : max_n;
     const int max_nn = max_m > max_n ? max_n : max_m;
     const int max_np = (max_nn + 1) & ~1;
-    if (max_mm > 16 * kRxG || max_np > 16 * kRxG || max_np < 2) return BSVD_ERR_UNSUPPORTED;
-    return p64 ? launch_rx<float, double, 16, 16>(batch, max_mm, max_np, A, M, N, LDA, S, U, LDU, V, LDV, tol,
-                                                  max_sweeps, info, rot, st, wl)
-               : launch_rx<float, float, 16, 16>(batch, max_mm, max_np, A, M, N, LDA, S, U, LDU, V, LDV, tol,
-                                                 max_sweeps, info, rot, st, wl);
+    if (max_mm > kRxRows || max_np > kRxRows || max_np < 2) return BSVD_ERR_UNSUPPORTED;
+    return p64 ? launch_rx<double>(batch, max_mm, max_np, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps, info, rot,
+                                   st, wl)
+               : launch_rx<float>(batch, max_mm, max_np, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps, info, rot,
+                                  st, wl);
 }
 
 }  // namespace bsvd
