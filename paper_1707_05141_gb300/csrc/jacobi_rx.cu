@@ -16,7 +16,7 @@
 // Bound by the W warps' dependent chain of a step (dot products, parameters, rotation, exchange); the V
 // warps fill the schedulers meanwhile.  With W and V in the same lanes, eight lanes a slot, both exchanged
 // through shared memory and the parameters computed eight times over, 1000 matrices of 127 x 100 took
-// 18.6 ms; it takes 13.1 ms here.
+// 18.6 ms; it takes 12.2 ms here.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -30,7 +30,11 @@ namespace {
 constexpr int kRxRows = 128, kRxSlots = 64;
 constexpr int kRxQuarter = 36, kRxLd = 4 * kRxQuarter;  // exchange area: strides of a lane's quarter column and of a
                                                         // slot: eight lanes' 16-byte accesses in distinct banks
-constexpr int kRxWThreads = 256, kRxThreads = kRxWThreads + 128;
+// threads of the form for up to SLOTS slots: W, V (a row each), both
+template <int SLOTS>
+struct RxThreads {
+    static constexpr int w = 4 * SLOTS, v = (2 * SLOTS + 31) / 32 * 32, all = w + v;
+};
 constexpr unsigned kRxFull = 0xffffffffu;
 
 struct RxShared {
@@ -47,11 +51,13 @@ template <int ID, int N>
 __device__ __forceinline__ void rx_wait() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
 template <int ID, int N>
 __device__ __forceinline__ void rx_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
-constexpr int kRxW = 1, kRxFullBar = 2, kRxEmptyBar = 4, kRxSweep = 6;
-__device__ __forceinline__ void rx_wait_full(int slot) { slot ? rx_wait<kRxFullBar + 1, kRxThreads>() : rx_wait<kRxFullBar, kRxThreads>(); }
-__device__ __forceinline__ void rx_wait_empty(int slot) { slot ? rx_wait<kRxEmptyBar + 1, kRxThreads>() : rx_wait<kRxEmptyBar, kRxThreads>(); }
-__device__ __forceinline__ void rx_arrive_full(int slot) { slot ? rx_arrive<kRxFullBar + 1, kRxThreads>() : rx_arrive<kRxFullBar, kRxThreads>(); }
-__device__ __forceinline__ void rx_arrive_empty(int slot) { slot ? rx_arrive<kRxEmptyBar + 1, kRxThreads>() : rx_arrive<kRxEmptyBar, kRxThreads>(); }
+constexpr int kRxW = 1, kRxFullBar = 2, kRxEmptyBar = 4, kRxSweep = 6, kRxRanks = 7;
+// (a barrier that both sides would reach with the same instruction is merged by the compiler into one block,
+// where W's and V's registers would be live together)
+template <int N> __device__ __forceinline__ void rx_wait_full(int slot) { slot ? rx_wait<kRxFullBar + 1, N>() : rx_wait<kRxFullBar, N>(); }
+template <int N> __device__ __forceinline__ void rx_wait_empty(int slot) { slot ? rx_wait<kRxEmptyBar + 1, N>() : rx_wait<kRxEmptyBar, N>(); }
+template <int N> __device__ __forceinline__ void rx_arrive_full(int slot) { slot ? rx_arrive<kRxFullBar + 1, N>() : rx_arrive<kRxFullBar, N>(); }
+template <int N> __device__ __forceinline__ void rx_arrive_empty(int slot) { slot ? rx_arrive<kRxEmptyBar + 1, N>() : rx_arrive<kRxEmptyBar, N>(); }
 
 __device__ __forceinline__ float2 rx_both(float x) { return make_float2(x, x); }
 
@@ -114,16 +120,17 @@ __device__ __forceinline__ bool rx_rotation(float al, float be, float ga, P tol,
 }  // namespace
 
 // P: precision of the rotation parameters and the rotation test (float, or double)
-template <typename P>
-__global__ void __launch_bounds__(kRxThreads, 1)
+template <typename P, int SLOTS>
+__global__ void __launch_bounds__(RxThreads<SLOTS>::all, 1)
     jacobi_rx_kernel(int batch, int max_mm, int max_np, float* const* A, const int* M, const int* N, const int* LDA,
                      float* const* Sout, float* const* U, const int* LDU, float* const* V, const int* LDV,
                      double tol_in, int max_sweeps, int* info, long long* rot_out, ItemList wl)
 {
+    constexpr int kW = RxThreads<SLOTS>::w, kAll = RxThreads<SLOTS>::all;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     RxShared& sh = *reinterpret_cast<RxShared*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool is_v = tid >= kRxWThreads;
+    const bool is_v = tid >= kW;
 
     for (int b = item_first(wl, batch); b >= 0; b = item_next(wl, batch, b)) {
         const int m = M[b], n = N[b], lda = LDA[b];
@@ -134,7 +141,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         const int ns = np / 2;      // slots of this matrix
         const bool wantU = U != nullptr, wantV = V != nullptr;
         const int ldu = wantU ? LDU[b] : 1, ldvo = wantV ? LDV[b] : 1;
-        const bool bad = m < 0 || n < 0 || mm > max_mm || np > max_np || mm > kRxRows || np > kRxRows ||
+        const bool bad = m < 0 || n < 0 || mm > max_mm || np > max_np || mm > kRxRows || np > 2 * SLOTS ||
                          lda < (m > 1 ? m : 1) || (wantU && ldu < (m > 1 ? m : 1)) ||
                          (wantV && ldvo < (n > 1 ? n : 1));
         if (bad) {
@@ -190,7 +197,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                 int rot_sweep = 0;
 #pragma unroll 1
                 for (int it = 0; it < ns; ++it) {
-                    if (accV && sent >= 2) rx_wait_empty(slot);
+                    if (accV && sent >= 2) rx_wait_empty<kAll>(slot);
                     // even step: positions 2s and 2s + 1; the right column moves one slot down
                     {
                         const float al = rx_dot(L, L), be = rx_dot(R, R), ga = rx_dot(L, R);
@@ -210,7 +217,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                         }
 #pragma unroll
                         for (int q = 0; q < 16; q += 2) out[q / 2] = make_float4(R[q].x, R[q].y, R[q + 1].x, R[q + 1].y);
-                        rx_wait<kRxW, kRxWThreads>();
+                        rx_wait<kRxW, kW>();
 #pragma unroll
                         for (int q = 0; q < 16; q += 2) {
                             const float4 v = from_up[q / 2];
@@ -247,7 +254,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                         }
 #pragma unroll
                         for (int q = 0; q < 16; q += 2) out1[q / 2] = make_float4(L[q].x, L[q].y, L[q + 1].x, L[q + 1].y);
-                        rx_wait<kRxW, kRxWThreads>();
+                        rx_wait<kRxW, kW>();
 #pragma unroll
                         for (int q = 0; q < 16; q += 2) {
                             const float4 v = from_dn[q / 2];
@@ -256,29 +263,29 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                         }
                     }
                     if (accV) {
-                        rx_arrive_full(slot);
+                        rx_arrive_full<kAll>(slot);
                         slot ^= 1;
                         ++sent;
                     }
                 }
                 if (lane == 0) sh.count[warp] = rot_sweep;
-                rx_wait<kRxW, kRxWThreads>();
+                rx_wait<kRxW, kW>();
                 rot_sweep = 0;
 #pragma unroll
-                for (int w = 0; w < kRxWThreads / 32; ++w) rot_sweep += sh.count[w];
+                for (int w = 0; w < kW / 32; ++w) rot_sweep += sh.count[w];
                 ++sweep;
                 total_rot += rot_sweep;
                 converged = rot_sweep == 0;
                 if (accV) {   // (a sweep of few columns has fewer double steps than the ring: both sides wait)
                     if (tid == 0) sh.more[sweep & 1] = !converged && sweep < sweeps_cap;
-                    rx_wait<kRxSweep, kRxThreads>();
+                    rx_wait<kRxSweep, kAll>();
                 }
                 if (converged) break;
-                rx_wait<kRxW, kRxWThreads>();   // the counts have been read
+                rx_wait<kRxW, kW>();   // the counts have been read
             }
             // the last double steps' "empty" arrivals
-            if (sent >= 2) rx_wait_empty(slot);
-            if (sent >= 1) rx_wait_empty(slot ^ 1);
+            if (sent >= 2) rx_wait_empty<kAll>(slot);
+            if (sent >= 1) rx_wait_empty<kAll>(slot ^ 1);
 
             // ---- sigma_j = ||w_j||; position p holds column p after an even number of sweeps, 2 NS - 1 - p
             // after an odd one (every sweep reverses the order) ----
@@ -289,7 +296,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                 if (colL < nn) sh.sig[colL] = sgL;
                 if (colR < nn) sh.sig[colR] = sgR;
             }
-            rx_wait<kRxW, kRxWThreads>();
+            rx_wait<kRxW, kW>();
             // ---- descending rank, ties in column order ----
             int rkL = 0, rkR = 0;
             for (int j = 0; j < nn; ++j) {
@@ -312,7 +319,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                 info[b] = !finite ? BSVD_INFO_NONFINITE : (converged ? sweep : BSVD_INFO_NOT_CONVERGED + sweep);
                 if (rot_out) rot_out[b] = total_rot;
             }
-            __syncthreads();   // the ranks are there
+            rx_arrive<kRxRanks, kAll>();   // the ranks are there
             if (uw) {
                 auto put = [&](const float2(&x)[16], int rk, float sg) {
                     if (rk < 0) return;
@@ -330,24 +337,25 @@ __global__ void __launch_bounds__(kRxThreads, 1)
             }
         } else {
             // ================================ V ================================
-            const int row = tid - kRxWThreads;
-            float v[2 * kRxSlots];   // row `row` of the column at each position
-            if (accV) {
+            const int row = tid - kW;
+            float v[2 * SLOTS];   // row `row` of the column at each position
 #pragma unroll
-                for (int p = 0; p < 2 * kRxSlots; ++p) v[p] = p == row ? 1.f : 0.f;
+            for (int p = 0; p < 2 * SLOTS; ++p) v[p] = p == row ? 1.f : 0.f;
+            {
                 int slot = 0, sweep = 0;
-                bool more = true;
+                // (not a branch around the loop: its second path would keep W's registers live beside V's)
+                bool more = accV;
                 while (more) {
 #pragma unroll 1
                     for (int it = 0; it < ns; ++it) {
                         // a double step in one pass: the odd step's pair (2p - 1, 2p) follows the even step's
                         // pair (2p, 2p + 1), so every result goes to a register whose old value has been used
-                        rx_wait_full(slot);
+                        rx_wait_full<kAll>(slot);
                         const float4* re = sh.ring[slot][0];
                         const float4* ro = sh.ring[slot][1];
                         float up = 0.f, oc = 1.f, os = 0.f;   // position 2p - 1 between the steps; its (c, s)
 #pragma unroll
-                        for (int p = 0; p < kRxSlots; p += 2) {
+                        for (int p = 0; p < SLOTS; p += 2) {
                             const float4 e = re[p / 2], o = ro[p / 2];
 #pragma unroll
                             for (int k = 0; k < 2; ++k) {
@@ -365,19 +373,19 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                                 os = k ? o.w : o.y;
                             }
                         }
-                        v[2 * kRxSlots - 1] = up;
-                        rx_arrive_empty(slot);
+                        v[2 * SLOTS - 1] = up;
+                        rx_arrive_empty<kAll>(slot);
                         slot ^= 1;
                     }
-                    rx_wait<kRxSweep, kRxThreads>();
+                    rx_wait<kRxSweep, kAll>();
                     ++sweep;
                     more = sh.more[sweep & 1] != 0;
                 }
             }
-            __syncthreads();   // the ranks are there
+            rx_wait<kRxRanks, kAll>();   // the ranks are there
             if (accV && row < nn) {
 #pragma unroll
-                for (int p = 0; p < 2 * kRxSlots; ++p) {
+                for (int p = 0; p < 2 * SLOTS; ++p) {
                     const int rk = p < np ? sh.rank[p] : -1;
                     if (rk >= 0) vw[(size_t)rk * ldvw + row] = v[p];
                 }
@@ -387,24 +395,27 @@ __global__ void __launch_bounds__(kRxThreads, 1)
     }
 }
 
-template <typename P>
+template <typename P, int SLOTS>
 static int launch_rx(int batch, int max_mm, int max_np, void* const* A, const int* M, const int* N, const int* LDA,
                      void* const* S, void* const* U, const int* LDU, void* const* V, const int* LDV, double tol,
                      int max_sweeps, int* info, long long* rot, cudaStream_t st, ItemList wl)
 {
-    auto kern = jacobi_rx_kernel<P>;
+    auto kern = jacobi_rx_kernel<P, SLOTS>;
     const size_t smem = sizeof(RxShared);
+    constexpr int threads = RxThreads<SLOTS>::all;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return BSVD_ERR_CUDA;
-    const int grid = item_grid(kern, kRxThreads, smem, wl, batch, st);
+    const int grid = item_grid(kern, threads, smem, wl, batch, st);
     if (grid == 0) return BSVD_ERR_CUDA;
-    kern<<<grid, kRxThreads, smem, st>>>(batch, max_mm, max_np, (float* const*)A, M, N, LDA, (float* const*)S,
-                                  (float* const*)U, LDU, (float* const*)V, LDV, tol, max_sweeps, info, rot, wl);
+    kern<<<grid, threads, smem, st>>>(batch, max_mm, max_np, (float* const*)A, M, N, LDA, (float* const*)S,
+                                      (float* const*)U, LDU, (float* const*)V, LDV, tol, max_sweeps, info, rot, wl);
     return cudaGetLastError() == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
 }
 
 // FP32 matrices with max(m, n) <= 128.  Returns BSVD_ERR_UNSUPPORTED for other shapes (the caller then takes
-// the shared tier).
+// the shared tier).  Up to 112 columns V leaves registers free and the V warps' work shrinks with the columns:
+// 1000 of
+// 127 x 100 take 13.1 ms with room for 128 columns (V spilling), 12.2 ms with 112.
 int launch_jacobi_rx(int batch, int max_m, int max_n, void* const* A, const int* M, const int* N, const int* LDA,
                      void* const* S, void* const* U, const int* LDU, void* const* V, const int* LDV, double tol,
                      int max_sweeps, int* info, long long* rot, cudaStream_t st, ItemList wl, bool p64)
@@ -413,10 +424,11 @@ int launch_jacobi_rx(int batch, int max_m, int max_n, void* const* A, const int*
     const int max_nn = max_m > max_n ? max_n : max_m;
     const int max_np = (max_nn + 1) & ~1;
     if (max_mm > kRxRows || max_np > kRxRows || max_np < 2) return BSVD_ERR_UNSUPPORTED;
-    return p64 ? launch_rx<double>(batch, max_mm, max_np, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps, info, rot,
-                                   st, wl)
-               : launch_rx<float>(batch, max_mm, max_np, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps, info, rot,
-                                  st, wl);
+#define BSVD_RX(P_, SLOTS_) \
+    launch_rx<P_, SLOTS_>(batch, max_mm, max_np, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps, info, rot, st, wl)
+    if (p64) return BSVD_RX(double, 64);
+    return max_np <= 96 ? BSVD_RX(float, 48) : (max_np <= 112 ? BSVD_RX(float, 56) : BSVD_RX(float, 64));
+#undef BSVD_RX
 }
 
 }  // namespace bsvd

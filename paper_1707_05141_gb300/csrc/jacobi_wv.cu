@@ -94,6 +94,7 @@ __device__ __forceinline__ float4 load4(const float* p, bool vec, int left)
     if (vec && left >= 4) return *reinterpret_cast<const float4*>(p);
     return make_float4(left > 0 ? p[0] : 0.f, left > 1 ? p[1] : 0.f, left > 2 ? p[2] : 0.f, left > 3 ? p[3] : 0.f);
 }
+__device__ __forceinline__ int again(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 __device__ __forceinline__ bool vec16(const void* p, int ld)
 {
     return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0;
@@ -111,7 +112,7 @@ __device__ __forceinline__ void bar_arrive(int threads)
 {
     asm volatile("bar.arrive %0, %1;" ::"n"(ID), "r"(threads) : "memory");
 }
-constexpr int kBarFull = 1, kBarEmpty = 3, kBarSweep = 5, kBarRed = 6;   // + ring slot for the first two
+constexpr int kBarFull = 1, kBarEmpty = 3, kBarSweep = 5, kBarRed = 6, kBarRanks = 7;   // + ring slot for the first two
 static_assert(kRing == 2, "two literal ids each");
 __device__ __forceinline__ void wait_full(int slot) { slot ? bar_wait<kBarFull + 1>(64) : bar_wait<kBarFull>(64); }
 __device__ __forceinline__ void wait_empty(int slot) { slot ? bar_wait<kBarEmpty + 1>(64) : bar_wait<kBarEmpty>(64); }
@@ -360,10 +361,17 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
         const bool sw = tr || pre;
         const bool accV = sw ? wantU : wantV;
         const float* a = A[b];
-        float* uw = sw ? (wantV ? V[b] : nullptr) : (wantU ? U[b] : nullptr);  // receives W / sigma
-        const int lduw = sw ? ldvo : ldu;
-        float* vw = sw ? (wantU ? U[b] : nullptr) : (wantV ? V[b] : nullptr);  // receives V (PRE: Q V_w)
-        const int ldvw = sw ? ldu : ldvo;
+        // the outputs' pointers and sizes are read where they are used: kept through the sweeps they would
+        // spill the columns
+        auto w_out = [&](int& ld) -> float* {   // receives W / sigma
+            if (!(sw ? wantV : wantU)) return nullptr;
+            ld = again((sw ? LDV : LDU) + b);
+            return (sw ? V : U)[b];
+        };
+        auto v_out = [&](int& ld) -> float* {   // receives V (PRE: Q V_w)
+            ld = again((sw ? LDU : LDV) + b);
+            return (sw ? U : V)[b];
+        };
 
         if constexpr (PRE) {
             if (pre) {
@@ -593,6 +601,7 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
                 }
             }
             const float sgL = dsqrt(na), sgR = dsqrt(nb);
+            const int nn = tr ? again(M + b) : again(N + b);
             if (warp == 0) {
                 sig_s[colL] = sgL;
                 sig_s[colR] = sgR;
@@ -619,7 +628,9 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
                     if (rot_out) rot_out[b] = total_rot;
                 }
             }
-            if (uw) {
+            int lduw = 0;
+            if (float* uw = w_out(lduw)) {
+                const int mm = tr ? again(N + b) : again(M + b);
                 const float iL = sgL > 0.f ? 1.f / sgL : 0.f, iR = sgR > 0.f ? 1.f / sgR : 0.f;
                 const float oL = __shfl_xor_sync(kFullWarp, iL, 16), oR = __shfl_xor_sync(kFullWarp, iR, 16);
                 const int ol = __shfl_xor_sync(kFullWarp, rkL, 16), or_ = __shfl_xor_sync(kFullWarp, rkR, 16);
@@ -637,14 +648,19 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
                 put(c2, h ? rkL : ol, h ? iL : oL);
                 put(c3, h ? rkR : or_, h ? iR : oR);
             }
-            __syncthreads();  // ranks (and, preconditioned, V in vs) are there
+            // V's output follows: preconditioned, the W warp waits for V in vs, else the V warp for the ranks
+            if (PRE && pre && accV)
+                bar_wait<kBarRanks>(32 * (WW + 1));
+            else
+                bar_arrive<kBarRanks>(32 * (WW + 1));
         } else {
             // ================================ V ================================
-            if (accV) {
-                float2 v[kCols];  // rows s and s + 32 of the column at each position
+            float2 v[kCols];  // rows s and s + 32 of the column at each position
 #pragma unroll
-                for (int p = 0; p < kCols; ++p) v[p] = make_float2(p == s ? 1.f : 0.f, p == s + 32 ? 1.f : 0.f);
-                bool more = true;
+            for (int p = 0; p < kCols; ++p) v[p] = make_float2(p == s ? 1.f : 0.f, p == s + 32 ? 1.f : 0.f);
+            {
+                // (not a branch around the loop: its second path would keep W's registers live beside V's)
+                bool more = accV;
                 while (more) {
                     // a double step in one pass over the pairs: the odd step's pair (2p - 1, 2p) follows
                     // the even step's pair (2p, 2p + 1), so every result goes to a register whose old
@@ -681,26 +697,28 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
                     }
                     more = more_s != 0;
                 }
-                if (PRE && pre) {
+            }
+            if (PRE && pre && accV) {
 #pragma unroll
-                    for (int p = 0; p < kCols; ++p) {
-                        vs[p * kLdV + s] = v[p].x;
-                        vs[p * kLdV + s + 32] = v[p].y;
-                    }
-                    __syncthreads();
-                } else {
-                    __syncthreads();
+                for (int p = 0; p < kCols; ++p) {
+                    vs[p * kLdV + s] = v[p].x;
+                    vs[p * kLdV + s + 32] = v[p].y;
+                }
+                __syncwarp();
+                bar_arrive<kBarRanks>(32 * (WW + 1));
+            } else {
+                bar_wait<kBarRanks>(32 * (WW + 1));
+                int ldvw = 0;
+                float* vw = accV ? v_out(ldvw) : nullptr;
+                const int nn = tr ? again(M + b) : again(N + b);
 #pragma unroll
-                    for (int p = 0; p < kCols; ++p) {
-                        const int rk = rank_s[p];
-                        if (rk >= 0) {
-                            if (s < nn) vw[(size_t)rk * ldvw + s] = v[p].x;
-                            if (s + 32 < nn) vw[(size_t)rk * ldvw + s + 32] = v[p].y;
-                        }
+                for (int p = 0; p < kCols; ++p) {
+                    const int rk = accV ? rank_s[p] : -1;
+                    if (rk >= 0) {
+                        if (s < nn) vw[(size_t)rk * ldvw + s] = v[p].x;
+                        if (s + 32 < nn) vw[(size_t)rk * ldvw + s + 32] = v[p].y;
                     }
                 }
-            } else {
-                __syncthreads();
             }
         }
 
@@ -753,6 +771,8 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
                     }
                 }
                 const int rkL = rank_s[cl], rkR = rank_s[cr];
+                int ldvw = 0;
+                float* vw = v_out(ldvw);
                 const bool vv = vec16(vw, ldvw);
 #pragma unroll
                 for (int k = 0; k < 32; k += 4) {
