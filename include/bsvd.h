@@ -476,6 +476,15 @@ int bsvd_host_qr(int dtype, int batch, int m, int n, const void* hA, void* hQ, v
                  void* workspace, size_t workspace_bytes, void* stream);
 
 /*
+ * bsvd_uniform_batch -- the DEVICE pointer and size arrays of a uniform batch whose matrix b starts
+ * b * stride_bytes after d_base: d_ptrs[b], d_m[b] = m, d_n[b] = n, d_ld[b] = ld, written by one small
+ * kernel on `stream` (a caller of a few small matrices otherwise spends most of a call filling them).
+ * Returns 0 or a negative argument code.
+ */
+int bsvd_uniform_batch(int batch, const void* d_base, long long stride_bytes, int m, int n, int ld, void** d_ptrs,
+                       int* d_m, int* d_n, int* d_ld, void* stream);
+
+/*
  * Diagnostics (outside the method; for tests and the benchmark).
  *
  * bsvd_philox_gauss -- for each of `count` counters (d_ctr: 4 x count words, DEVICE) the

@@ -101,6 +101,8 @@ def lib() -> ctypes.CDLL:
             L.bsvd_host_qr.argtypes = [i, i, i, i, p, p, p, p, i, p, ctypes.c_size_t, p]
             L.bsvd_philox_gauss.restype = i
             L.bsvd_philox_gauss.argtypes = [i, p, ctypes.c_ulonglong, p, p, p, p]
+            L.bsvd_uniform_batch.restype = i
+            L.bsvd_uniform_batch.argtypes = [i, p, ll, i, i, i, p, p, p, p, p]
             L.bsvd_fma_probe.restype = ctypes.c_longlong
             L.bsvd_fma_probe.argtypes = [i, i, i, p, p]
             L.batched_rsvd.restype = i
@@ -235,12 +237,22 @@ class Batch:
         bsz, cols, ld = t.shape
         m = ld if m is None else m
         n = cols if n is None else n
-        es = t.element_size()
-        base = int(t.data_ptr())
-        dev = t.device
-        ptrs = base + torch.arange(bsz, device=dev, dtype=torch.int64) * (cols * ld * es)
-        full = lambda v: torch.full((bsz,), int(v), device=dev, dtype=torch.int32)
-        return cls(ptrs, full(m), full(n), full(ld), t.dtype, m, n, keep=(t,))
+        if max(abs(int(m)), abs(int(n)), ld) > 0x7fffffff:
+            raise OverflowError("Batch.uniform: sizes are 32-bit integers")
+        # the four arrays by one kernel: a call on a few small matrices makes up to four batches, and
+        # filling them by tensor operations (24 launches) took most of its time (16 of 33 x 20,
+        # singular values and vectors: 323 -> 169 us)
+        ptrs = torch.empty(bsz, device=t.device, dtype=torch.int64)
+        sizes = torch.empty((3, bsz), device=t.device, dtype=torch.int32)
+        args = (bsz, t.data_ptr(), cols * ld * t.element_size(), int(m), int(n), ld, ptrs.data_ptr(),
+                sizes.data_ptr(), sizes.data_ptr() + 4 * bsz, sizes.data_ptr() + 8 * bsz)
+        if t.device.index == torch.cuda.current_device():
+            rc = lib().bsvd_uniform_batch(*args, torch.cuda.current_stream().cuda_stream)
+        else:
+            with torch.cuda.device(t.device):
+                rc = lib().bsvd_uniform_batch(*args, torch.cuda.current_stream().cuda_stream)
+        _check("bsvd_uniform_batch", rc)
+        return cls(ptrs, *sizes.unbind(), t.dtype, m, n, keep=(t,))
 
     @classmethod
     def packed(cls, flat, offsets, m, n, ld=None):

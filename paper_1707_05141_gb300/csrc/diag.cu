@@ -56,6 +56,18 @@ __global__ void __launch_bounds__(256) fma_probe_kernel(int iters, T x, T y, T* 
     out[blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
+// pointer and size arrays of a uniform batch, one thread per matrix
+__global__ void uniform_batch_kernel(int batch, unsigned char* base, long long stride, int m, int n, int ld,
+                                     void** ptrs, int* M, int* N, int* LD)
+{
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= batch) return;
+    ptrs[b] = base + (long long)b * stride;
+    M[b] = m;
+    N[b] = n;
+    LD[b] = ld;
+}
+
 }  // namespace bsvd
 
 using namespace bsvd;
@@ -70,6 +82,21 @@ int bsvd_philox_gauss(int count, const unsigned* d_ctr, unsigned long long seed,
     if (!d_ctr) return -2;
     cudaStream_t st = (cudaStream_t)stream;
     philox_gauss_kernel<<<(count + 127) / 128, 128, 0, st>>>(count, d_ctr, seed, d_words, d_gauss, d_gauss64);
+    return cudaGetLastError() == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
+}
+
+int bsvd_uniform_batch(int batch, const void* d_base, long long stride_bytes, int m, int n, int ld, void** d_ptrs,
+                       int* d_m, int* d_n, int* d_ld, void* stream)
+{
+    if (batch < 0) return -1;
+    if (batch == 0) return BSVD_SUCCESS;
+    if (!d_base && stride_bytes != 0) return -2;
+    if (!d_ptrs) return -7;
+    if (!d_m) return -8;
+    if (!d_n) return -9;
+    if (!d_ld) return -10;
+    uniform_batch_kernel<<<(batch + 127) / 128, 128, 0, (cudaStream_t)stream>>>(
+        batch, (unsigned char*)const_cast<void*>(d_base), stride_bytes, m, n, ld, d_ptrs, d_m, d_n, d_ld);
     return cudaGetLastError() == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
 }
 
