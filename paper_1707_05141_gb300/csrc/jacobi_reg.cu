@@ -48,6 +48,7 @@
 
 #include "common.cuh"
 #include "launch.cuh"
+#include "rnmath.cuh"
 
 namespace bsvd {
 
@@ -73,6 +74,12 @@ __global__ void __launch_bounds__(NS * PARTS, MINB)
     // rotation parameters (zeta, t, c, s) and the rotation test in the working precision, or in
     // FP64 for FP32 data (P64): the Gram entries are summed in T, then promoted
     typedef typename std::conditional<P64, double, T>::type P;
+    // carried norms leave one sum per step, and the chain of the parameters behind it shows: branch-free
+    // ones (rnmath.cuh) and no parameters in a step that rotates nothing: 500 / 10 000 preconditioned 32 x 32
+    // matrices 0.208 / 1.30 -> 0.189 / 1.24 ms.
+    // Where all three sums are formed, they hide the chain and the built-in operations' fewer
+    // instructions are 2 to 9 % faster.
+    constexpr bool RN = CARRY && !P64 && sizeof(T) == 4;
 
     __shared__ Red3<T> red[2][NW > 1 ? NW : 1][32];
     __shared__ T sig_s[NC];
@@ -321,7 +328,24 @@ __global__ void __launch_bounds__(NS * PARTS, MINB)
                 const bool rot = !(odd && s == NS - 1) && alpha > P(0) && beta > P(0) &&
                                  off_diagonal_large(alpha, beta, gamma, tol);
                 P tth = P(0), cth = P(1);
-                if (rot) {
+                T kL = T(1), kR = T(1);   // FAST: d_j / d_i and d_i / d_j
+                if (RN && !__any_sync(0xffffffffu, rot)) {
+                    // (most steps of the last sweeps)
+                } else if constexpr (RN) {
+                    // every lane, without branches (a lane that does not rotate drops the result): the
+                    // correctly rounded operations of the branches below, the same numbers
+                    kL = dR * rn_rcp(dL);   // (2^-33 < d <= 1)
+                    kR = dL * rn_rcp(dR);
+                    const float d = beta - alpha, g2 = 2.f * gamma;
+                    const float ad = fabsf(d), ag = fabsf(g2);
+                    const float sl = pow2_scale(ad > ag ? ad : ag);
+                    const float dn = ad * sl, gn = g2 * sl;   // the larger is in [1, 2)
+                    const float den = dn + rn_sqrt(fmaf(dn, dn, gn * gn));
+                    float t = rn_div(gn, den);
+                    if (__any_sync(0xffffffffu, rot && !(fabsf(gn) >= 0x1p-100f && den < 8.f))) t = gn / den;
+                    tth = rot ? (d >= 0.f ? t : -t) : 0.f;
+                    cth = rn_rsqrt12(fmaf(tth, tth, 1.f));
+                } else if (rot) {
                     tth = jacobi_t(alpha, beta, gamma);
                     cth = drsqrt(P(1) + tth * tth);
                 }
@@ -333,8 +357,12 @@ __global__ void __launch_bounds__(NS * PARTS, MINB)
                 } else if (FAST) {
                     // scale ratios from the current scales (correctly rounded reciprocals), so that
                     // their rounding does not accumulate over the rotations of a sweep
-                    const T mL = -T(tth) * (dR * rcp_rn(dL));  // -t d_j / d_i
-                    const T mR = T(tth) * (dL * rcp_rn(dR));   //  t d_i / d_j
+                    if constexpr (!RN) {
+                        kL = dR * rcp_rn(dL);
+                        kR = dL * rcp_rn(dR);
+                    }
+                    const T mL = -T(tth) * kL;  // -t d_j / d_i
+                    const T mR = T(tth) * kR;   //  t d_i / d_j
 #pragma unroll
                     for (int k = 0; k < RA; ++k) {
                         const T x = aL[k], y = aR[k];
@@ -374,8 +402,7 @@ __global__ void __launch_bounds__(NS * PARTS, MINB)
                     nL = tnL;
                     nR = tnR;
                     if (rot) {
-                        const T tg = T(tth * gamma);
-                        const T aN = tnL - tg, bN = tnR + tg;
+                        const T aN = fma(-T(tth), T(gamma), tnL), bN = fma(T(tth), T(gamma), tnR);
                         nL = aN < T(0.25) * tnL ? T(-1) : aN;
                         nR = bN < T(0.25) * tnR ? T(-1) : bN;
                     }
@@ -563,6 +590,22 @@ __global__ void __launch_bounds__(NS * PARTS, MINB)
     }
 }
 
+// The plain 32-slot FP32 variants have both forms: the one above (two or four warps with half or a quarter
+// of the rows of W and V each) and jacobi_wv.cu's (half as many W warps with all the columns in half the
+// lanes, V elsewhere).  Up to two matrices per SM a step's latency is what counts, and it is shorter
+// above: 54 x 45, 16 / 304 matrices with U and V 0.80 / 0.84 ms against 0.86 / 0.95.  Beyond, the issue
+// slots count: 608 matrices 1.05 against 1.02 ms, 8000 10.9 against 9.6 (120 x 50: 1.39 against 0.96 and
+// 17.4 against 11.6).  Without U and V two parts have nothing to keep out of W's warps: 0.83 against 0.88 ms
+// at 608, 8.25 against 8.22 at 8000.  (Preconditioned or with FP64 parameters, jacobi_wv.cu is faster
+// from 16 matrices on.)
+static bool use_wv(int parts, bool vectors, int batch)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return batch > 2 * sms && (parts == 4 || vectors);
+}
+
 template <typename T, int NS, int PARTS, int RA, int RV, int MINB, bool FAST, bool PRE, bool P64, bool CARRY>
 static int launch_reg(int batch, void* const* A, const int* M, const int* N, const int* LDA, void* const* S,
                       void* const* U, const int* LDU, void* const* V, const int* LDV, double tol, int max_sweeps,
@@ -570,10 +613,14 @@ static int launch_reg(int batch, void* const* A, const int* M, const int* N, con
 {
     if constexpr (sizeof(T) == 4 && NS == 32 && RA == 32 && FAST) {
         // 32 slots, parts of 32 rows: W and V in separate warps (jacobi_wv.cu; the same sums and
-        // rotations, bit for bit: 20 000 preconditioned 64 x 64 matrices 18.6 -> 13.8 ms)
-        return launch_jacobi_wv(PARTS == 4, PRE, P64, CARRY, batch, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps,
-                                info, rot, st, wl);
-    } else {
+        // rotations, bit for bit: 20 000 preconditioned 64 x 64 matrices 18.6 -> 13.8 ms).  A W warp there
+        // has twice the columns and half the steps' barriers of a warp here, so its step takes longer
+        // and more matrices fit an SM.
+        if (PRE || P64 || use_wv(PARTS, U || V, batch))
+            return launch_jacobi_wv(PARTS == 4, PRE, P64, CARRY, batch, A, M, N, LDA, S, U, LDU, V, LDV, tol,
+                                    max_sweeps, info, rot, st, wl);
+    }
+    if constexpr (!(sizeof(T) == 4 && NS == 32 && RA == 32 && FAST && (PRE || P64))) {
         auto kern = jacobi_reg_kernel<T, NS, PARTS, RA, RV, MINB, FAST, PRE, P64 && sizeof(T) == 4, CARRY>;
         const int grid = item_grid(kern, NS * PARTS, 0, wl, batch, st);
         if (grid == 0) return BSVD_ERR_CUDA;
@@ -581,6 +628,7 @@ static int launch_reg(int batch, void* const* A, const int* M, const int* N, con
                                           (T* const*)V, LDV, tol, max_sweeps, info, rot, wl);
         return cudaGetLastError() == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
     }
+    return BSVD_ERR_UNSUPPORTED;  // (not reached)
 }
 
 // Register-tier variants (slots, row parts, A rows per lane, V rows per lane, resident CTAs, scaled

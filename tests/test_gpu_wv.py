@@ -147,3 +147,35 @@ def test_branch_free_operations_are_correctly_rounded(tmp_path):
     out = (ctypes.c_ulonglong * 4)()
     assert ctypes.CDLL(str(so)).rn_check(out) == 0
     assert list(out) == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("vectors", [True, False])
+@pytest.mark.parametrize("m,n,carried", [(54, 45, False), (64, 64, True), (37, 64, False), (120, 50, False)])
+def test_small_and_large_batches_agree(bs, m, n, carried, vectors):
+    """The plain 32-slot variants take a batch of more than two matrices per SM to the form with W and V in
+    separate warps and a smaller one to the form with both in the same: the same numbers, bit for bit."""
+    per = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    variant = 0
+    for k in range(1, bs.jacobi_variants(bs.F32, m, n, bs.TIER_REGISTER) + 1):
+        d = bs.jacobi_variant_desc(bs.F32, m, n, k)
+        if carried and d["carried_norms"] and not d["qr_precond"] and d["slots"] == 32:
+            variant = k
+    assert bool(variant) == carried
+    a = torch.randn((per + 1, n, m), device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    a *= torch.exp(-torch.arange(n, device="cuda") / 8.0)[None, :, None]
+    k = min(m, n)
+
+    def run(x):
+        b = x.shape[0]
+        s, u, v = (torch.zeros(z, device="cuda") for z in ((b, 1, k), (b, k, m), (b, k, n)))
+        info = torch.zeros(b, dtype=torch.int32, device="cuda")
+        rot = torch.zeros(b, dtype=torch.int64, device="cuda")
+        U = bs.Batch.uniform(u, m, k) if vectors else None
+        V = bs.Batch.uniform(v, n, k) if vectors else None
+        bs.batched_svd_jacobi(bs.Batch.uniform(x, m, n), bs.Batch.uniform(s, k, 1), U, V, info, rot,
+                              tier=bs.TIER_REGISTER | (variant << 8))
+        return s, u, v, info, rot
+
+    large, small, last = run(a), run(a[:per].contiguous()), run(a[per:].contiguous())
+    for x, y, z in zip(large, small, last):
+        assert torch.equal(x, torch.cat([y, z]))
