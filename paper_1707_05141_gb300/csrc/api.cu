@@ -105,6 +105,10 @@ int batched_qr(int dtype, int batch, int max_m, int max_n, void* const* dA, cons
     if (max_n == 0) max_n = 1;
     if (max_m == 0) max_m = 1;
     cudaStream_t st = (cudaStream_t)stream;
+    if (dtype == BSVD_F32) {
+        const int rc = launch_qr_wy(batch, max_m, max_n, dA, d_m, d_n, d_lda, dQ, d_ldq, dR, d_ldr, d_info, st);
+        if (rc != BSVD_ERR_UNSUPPORTED) return rc;
+    }
     return dtype == BSVD_F32 ? launch_qr<float>(batch, max_m, max_n, dA, d_m, d_n, d_lda, dQ, d_ldq, dR, d_ldr, d_info, st)
                              : launch_qr<double>(batch, max_m, max_n, dA, d_m, d_n, d_lda, dQ, d_ldq, dR, d_ldr, d_info, st);
 }

@@ -15,6 +15,9 @@ int launch_qr(int batch, int max_m, int max_n, void* const* A, const int* M, con
               void* const* Q, const int* LDQ, void* const* R, const int* LDR, int* info, cudaStream_t st,
               ItemList wl = all_items(), bool r_transposed = false,  // r_transposed: R^T written to R
               const int* a_trans = nullptr);  // a_trans[b] != 0: factor A^T (stored n x m, ld LDA)
+// the blocked form for wider FP32 matrices (qr_wy.cu); BSVD_ERR_UNSUPPORTED where launch_qr is to be used
+int launch_qr_wy(int batch, int max_m, int max_n, void* const* A, const int* M, const int* N, const int* LDA,
+                 void* const* Q, const int* LDQ, void* const* R, const int* LDR, int* info, cudaStream_t st);
 template <typename T>
 int launch_jacobi_reg(int batch, int max_m, int max_n, int variant, void* const* A, const int* M, const int* N,
                       const int* LDA, void* const* S, void* const* U, const int* LDU, void* const* V, const int* LDV,
