@@ -24,7 +24,7 @@
 // 480 of them exchange, 400 parameters, 260 dot products; 12 warps in 168 registers each on an SM).
 // Measured (GB300, before -> after): 20 000 preconditioned 64 x 64 matrices 18.6 -> 13.8 ms; 500 of
 // 512 x 512 by the block tier, whose inner SVDs these are, 230 -> 212 ms; a depth-12 basis tree (128-row
-// form) 16.0 -> 13.0 ms.
+// form) 16.0 -> 12.4 ms.
 #include <cuda_runtime.h>
 
 #include <type_traits>
@@ -197,18 +197,19 @@ __device__ __forceinline__ unsigned wv_step(float2 (&c0)[16], float2 (&c1)[16], 
         tnL = q.dL * q.dL * sa;
         tnR = q.dR * q.dR * sb;
     }
-    // rotation of the pair, in the unscaled frame; the wrap slot idles on odd steps.  With carried norms the
-    // parameters are computed by every lane without branches (a lane that does not rotate drops them),
-    // so that the reciprocals and the test run under the dot product and the cosine under the exchange;
-    // with three sums a step the built-in operations' fewer instructions are faster (20 000 of 54 x 45:
-    // 23.4 against 22.6 ms).
+    // rotation of the pair, in the unscaled frame; the wrap slot idles on odd steps.  With carried norms or
+    // two W warps the parameters are computed by every lane without branches (a lane that does not
+    // rotate drops them), so that the reciprocals and the test run under the dot product and the cosine
+    // under the exchange (128 rows: a depth-12 basis tree 12.9 -> 12.4 ms);
+    // with one warp and three sums a step the built-in operations' fewer instructions are faster
+    // (20 000 of 54 x 45: 23.4 against 22.6 ms).
     const P alpha = CARRY ? P(tnL) : P(q.dL) * P(q.dL) * P(sa);
     const P beta = CARRY ? P(tnR) : P(q.dR) * P(q.dR) * P(sb);
     const P gamma = P(q.dL) * P(q.dR) * P(sc);
     const bool rot = !(ODD && lane == 31) && alpha > P(0) && beta > P(0) && off_diagonal_large(alpha, beta, gamma, tol);
     const unsigned rots = __ballot_sync(kFullWarp, rot);
     float mL = 0.f, mR = 0.f, cth = 1.f, tth = 0.f;
-    if constexpr (P64 || !CARRY) {
+    if constexpr (P64 || (!CARRY && WW == 1)) {
         if (rot) {
             const P t = jacobi_t(alpha, beta, gamma);
             tth = float(t);

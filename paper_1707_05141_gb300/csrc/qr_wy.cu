@@ -14,8 +14,8 @@
 // The order of the sums differs from qr_kernel's, so the randomized SVD, whose singular vectors move
 // with the last bit of R, keeps that one.
 // Measured (GB300, before -> here): 2000 matrices of 250 x 149 7.54 -> 3.62 ms, of 180 x 80 3.08 -> 1.64,
-// 20 of 250 x 149 0.54 -> 0.26.  One CTA per SM; the panels' chain of barriers (about a third) and the
-// shared-memory loads of the updates bound it.
+// 20 of 250 x 149 0.54 -> 0.26.  One CTA per SM; by its code, the panels' chain of
+// barriers and the shared-memory loads of the updates bound it.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
