@@ -805,12 +805,14 @@ __global__ void __launch_bounds__(256, 3) qw_apply_kernel(int p, int trans, int 
     auto stage = [&](int s) {
         const int s0 = s * SR;
         constexpr int PC = SR / VE;   // vectors per column
-        auto column = [&](T* dst, const T* src, bool vec, int left) {   // one vector; left: valid elements
+        // one vector; left: valid elements; base: the operand's first element, which a vector without valid elements
+        // names as its source (16-byte aligned where vec is set; the copy wants that of a source it does not read, too)
+        auto column = [&](T* dst, const T* src, const T* base, bool vec, int left) {
             if (vec) {
                 left = left < 0 ? 0 : (left > VE ? VE : left);
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
                                  (unsigned)__cvta_generic_to_shared(dst)),
-                             "l"(left > 0 ? src : X), "r"(left * (int)sizeof(T))
+                             "l"(left > 0 ? src : base), "r"(left * (int)sizeof(T))
                              : "memory");
             } else {
 #pragma unroll
@@ -820,8 +822,8 @@ __global__ void __launch_bounds__(256, 3) qw_apply_kernel(int p, int trans, int 
 #pragma unroll 4
         for (int e = tid; e < kPw * PC; e += 256) {
             const int c = e / PC, r = (e % PC) * VE, left = rows - (s0 + r);
-            column(Vs + c * LD + r, V + (size_t)c * mm + s0 + r, vv, c < vcols ? left : 0);
-            column(Cs + c * LD + r, C + (size_t)c * ldc + s0 + r, vc, c < ncol ? left : 0);
+            column(Vs + c * LD + r, V + (size_t)c * mm + s0 + r, V, vv, c < vcols ? left : 0);
+            column(Cs + c * LD + r, C + (size_t)c * ldc + s0 + r, C, vc, c < ncol ? left : 0);
         }
         asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
         if (s == 0) {   // R's entries of the panel's first rows

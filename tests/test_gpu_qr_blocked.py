@@ -1,0 +1,54 @@
+"""GPU parity: blocked QRs whose copies in the workspace and whose Q differ in alignment."""
+import numpy as np
+import pytest
+
+from parity import gate
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def blocked_qr(mats, ldq=None):
+    """Q, R (64 bits) and info of a batch of matrices of one type; column j of Q starts on a multiple of ldq[b]
+    elements after a 16-byte boundary."""
+    import paper_1707_05141_gb300 as bs
+    bs.build()
+    m, n = (np.array([a.shape[i] for a in mats], np.int32) for i in (0, 1))
+    ldq = m if ldq is None else np.asarray(ldq, np.int32)
+
+    def pack(ld, cols):
+        off = np.concatenate([[0], np.cumsum((ld.astype(np.int64) * np.maximum(cols, 1) + 3) // 4 * 4)])
+        return np.zeros(int(off[-1]) + 4, mats[0].dtype), off[:-1]
+
+    (fa, oa), (fq, oq), (fr, orr) = pack(m, n), pack(ldq, n), pack(n, n)
+    for a, o in zip(mats, oa):
+        fa[o:o + a.size] = a.T.reshape(-1)
+    ta, tq, tr = (torch.from_numpy(x).cuda() for x in (fa, fq, fr))
+    A, Q, R = bs.Batch.packed(ta, oa, m, n), bs.Batch.packed(tq, oq, m, n, ldq), bs.Batch.packed(tr, orr, n, n)
+    info = torch.full((len(mats),), 7, dtype=torch.int32, device="cuda")
+    ws = torch.empty(bs.batched_qr_blocked_workspace(A), dtype=torch.uint8, device="cuda")
+    bs.batched_qr_blocked(A, Q, R, info, ws)
+    torch.cuda.synchronize()
+    hq, hr = tq.cpu().numpy().astype(np.float64), tr.cpu().numpy().astype(np.float64)
+    q = [np.stack([hq[o + j * l:][:mm] for j in range(nn)], 1) for o, l, mm, nn in zip(oq, ldq, m, n)]
+    r = [hr[o:o + nn * nn].reshape(nn, nn).T for o, nn in zip(orr, n)]
+    return q, r, info.cpu().numpy()
+
+
+# (the workspace holds matrix b at b max_m max_n elements: misaligned for an odd product and an odd b, while
+# Q's columns are 16-byte aligned, so V and C of a block reflector are copied by different means)
+@pytest.mark.parametrize("dt,shapes", [(np.float32, [(257, 65), (256, 64), (256, 33), (252, 65)]),
+                                       (np.float32, [(2001, 601), (2001, 601)]),
+                                       (np.float32, [(33, 33), (32, 1), (29, 29)]),
+                                       (np.float64, [(131, 33), (128, 33), (130, 1)])])
+def test_aligned_q_beside_unaligned_workspace(dt, shapes):
+    rng = np.random.default_rng(2)
+    mats = [rng.standard_normal(s).astype(dt) for s in shapes]
+    assert max(s[0] for s in shapes) * max(s[1] for s in shapes) % 2 == 1
+    q, r, info = blocked_qr(mats, [(s[0] + 3) // 4 * 4 for s in shapes])
+    assert (info == 0).all()
+    for a, qq, rr in zip(mats, q, r):
+        a = a.astype(np.float64)
+        assert np.abs(qq.T @ qq - np.eye(a.shape[1])).max() <= gate(dt), a.shape
+        assert np.linalg.norm(a - qq @ rr) <= gate(dt) * np.linalg.norm(a), a.shape
+        assert not np.tril(rr, -1).any()
