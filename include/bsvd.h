@@ -127,7 +127,8 @@ int batched_qr_blocked_max_rows(int dtype);
  *   dU[b]  (out) m x k left singular vectors, ld d_ldu[b] >= m; dU may be NULL.  A column whose
  *                singular value is zero is written as zeros.
  *   dV[b]  (out) n x k right singular vectors (accumulated rotations), ld d_ldv[b] >= n; dV may
- *                be NULL, which also skips the accumulation.
+ *                be NULL, which also skips the accumulation.  A null entry of dU or dV: that
+ *                matrix's factor is not written.
  *   tol    rotation threshold: pair (i, j) is rotated only when
  *          |a_i . a_j| > tol * ||a_i|| ||a_j||.  tol <= 0 selects sqrt(max(m, n)) * u with u the
  *          unit roundoff of dtype (2^-24 or 2^-53).

@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(RxThreads<SLOTS>::all, 1)
                 }
             }
             rx_wait<kRxRanks, kAll>();   // the ranks are there
-            if (accV && row < nn) {
+            if (accV && vw && row < nn) {   // (a null entry of the pointer array: that matrix's V is not written)
 #pragma unroll
                 for (int p = 0; p < 2 * SLOTS; ++p) {
                     const int rk = p < np ? sh.rank[p] : -1;

@@ -717,7 +717,7 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
                 const int nn = tr ? again(M + b) : again(N + b);
 #pragma unroll
                 for (int p = 0; p < kCols; ++p) {
-                    const int rk = accV ? rank_s[p] : -1;
+                    const int rk = vw ? rank_s[p] : -1;   // (null also where the pointer array has a null entry)
                     if (rk >= 0) {
                         if (s < nn) vw[(size_t)rk * ldvw + s] = v[p].x;
                         if (s + 32 < nn) vw[(size_t)rk * ldvw + s + 32] = v[p].y;
@@ -774,9 +774,9 @@ __global__ void __launch_bounds__(32 * (WW + 1), MINB)
                         vR[k + 3] = fmaf(dr, x.w, vR[k + 3]);
                     }
                 }
-                const int rkL = rank_s[cl], rkR = rank_s[cr];
                 int ldvw = 0;
                 float* vw = v_out(ldvw);
+                const int rkL = vw ? rank_s[cl] : -1, rkR = vw ? rank_s[cr] : -1;
                 const bool vv = vec16(vw, ldvw);
 #pragma unroll
                 for (int k = 0; k < 32; k += 4) {
