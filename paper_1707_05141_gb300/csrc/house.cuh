@@ -6,6 +6,30 @@
 
 namespace bsvd {
 
+// Scaling of a panel's columns by powers of two.  The register panels (qr_wy.cu, qr_blocked.cu) multiply the raw
+// pivot column with the others, products of the size of two columns' norms multiplied; with every column's largest
+// magnitude in [1, 2) they stay in the type's range wherever the columns are.  (Unscaled, FP32 columns of 1e21 and
+// 1e17 gave NaN, and columns of 1e-26 and 1e-17 an error of 5e-4.)  Every operation on a column scales with it and
+// the reflectors do not depend on it, so inside the range the results are the same numbers; R's entries are scaled back.
+
+// magnitude as an integer that orders like it (FP64: its upper word)
+__device__ __forceinline__ unsigned magnitude(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned magnitude(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// largest magnitude of a warp's values
+template <typename T, int N>
+__device__ __forceinline__ unsigned warp_magnitude(const T (&x)[N])
+{
+    unsigned g = 0;
+#pragma unroll
+    for (int t = 0; t < N; ++t) g = max(g, magnitude(x[t]));
+    return __reduce_max_sync(0xffffffffu, g);
+}
+
+// the power of two for a magnitude (clamped, so that its inverse is a normal number too)
+__device__ __forceinline__ float column_scale(unsigned g, float) { return pow2_scale(__uint_as_float(g)); }
+__device__ __forceinline__ double column_scale(unsigned g, double) { return pow2_scale(__hiloint2double((int)g, 0)); }
+
 // The reflector of column i, formed by one warp: v = house(S(i:m, i)) (norm by a warp shuffle
 // reduction), stored normalised so that the reflector is I - 2 v v^T in S(i:m, i), and
 // R(i, i) = -sign(x_0) ||x|| in diag[i].  A zero column gives v = 0 (identity reflector), R(i, i) = 0.

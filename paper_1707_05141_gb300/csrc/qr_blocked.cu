@@ -599,6 +599,8 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
     __shared__ T pub[2][RPL * 32];            // the pivot column of this CTA's rows
     __shared__ T xch[2][kClusterMax][kPw];    // the CTAs' partial products with the pivot
     __shared__ T row[2][kPw];                 // row c of the panel
+    __shared__ unsigned mags[kClusterMax][kPw];   // the CTAs' largest magnitudes of the columns
+    __shared__ T back[kPw];                   // powers of two that the columns' entries of R are multiplied by
     __shared__ T Gs[kPw][kPw + 1], Ts[kPw][kPw + 1];   // V^T V (above the diagonal) and T (row i, column c)
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
@@ -620,6 +622,33 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
             const int c = 2 * warp + q, r = lane + 32 * t;
             x[q][t] = (owner && c < vcols && r < nr) ? X[(size_t)c * mm + r] : T(0);
         }
+    // the columns scaled (house.cuh) by their largest magnitude in all of the cluster's rows
+    unsigned mag[2] = {0, 0};
+    if (owner) {
+        mag[0] = warp_magnitude(x[0]);
+        mag[1] = warp_magnitude(x[1]);
+    }
+    if (cs > 1) {
+        cluster.sync();                       // every CTA of the cluster runs before the first push
+        if (owner && lane < cs) {
+            unsigned* g = cluster.map_shared_rank(&mags[rank][2 * warp], lane);
+            g[0] = mag[0];
+            g[1] = mag[1];
+        }
+        cluster.sync();
+        if (owner)
+            for (int k = 0; k < cs; ++k) {
+                mag[0] = max(mag[0], mags[k][2 * warp]);
+                mag[1] = max(mag[1], mags[k][2 * warp + 1]);
+            }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const T sc = column_scale(mag[q], T(0));
+        if (owner && lane == 0) back[2 * warp + q] = T(1) / sc;
+#pragma unroll
+        for (int t = 0; t < RPL; ++t) x[q][t] *= sc;
+    }
     if (warp == 0) {
 #pragma unroll
         for (int t = 0; t < RPL; ++t) pub[0][lane + 32 * t] = x[0][t];
@@ -632,8 +661,7 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
         for (int e = 0; e < k; ++e) s = fma(Ts[lane][e], Gs[e][k], s);
         if (lane <= k) Ts[lane][k] = lane == k ? T(2) : T(-2) * s;
     };
-    if (cs > 1) cluster.sync();               // every CTA of the cluster runs before the first push
-    else __syncthreads();
+    __syncthreads();
     for (int c = 0; c < vcols; ++c) {
         const int buf = c & 1;
         if (owner) {
@@ -690,7 +718,7 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
                 w[q] = j > c ? T(-2) * z : T(0);
                 if (j < c && rank == 0 && lane == 0) Gs[j][c] = z;
             }
-            if (rank == 0 && warp == 0 && lane == 0) rd[c] = alpha > T(0) ? -sa : T(0);
+            if (rank == 0 && warp == 0 && lane == 0) rd[c] = alpha > T(0) ? -sa * back[c] : T(0);
 #pragma unroll
             for (int t = 0; t < RPL; ++t) {
                 T v = pub[buf][lane + 32 * t] * inv;
@@ -718,7 +746,7 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
 #pragma unroll
             for (int t = 0; t < RPL; ++t) {
                 const int c = 2 * warp + q, r = lane + 32 * t;
-                if (c < vcols && r < nr) X[(size_t)c * mm + r] = x[q][t];
+                if (c < vcols && r < nr) X[(size_t)c * mm + r] = t == 0 && rank == 0 && lane < c ? x[q][t] * back[c] : x[q][t];
             }
     } else if (rank == 0) {
         t_column(vcols - 1);

@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "house.cuh"
 #include "launch.cuh"
 
 namespace bsvd {
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ float pub[2][RPL * 32];          // the pivot column, zero above its row
     __shared__ float sum[2][kPw], row[2][kPw];  // its products with the panel's columns; its row of the panel
     __shared__ float Gs[kPw][kLdT], Ts[kPw][kLdT];   // V^T V (above the diagonal) and T (row i, column c)
-    __shared__ float diag[kPw];
+    __shared__ float diag[kPw], back[kPw];      // R's diagonal; powers of two that a column's entries of R are multiplied by
 
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m = M[b], n = N[b], lda = LDA[b];
@@ -226,6 +227,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int c = 2 * warp + q, r = lane + 32 * t;
                 x[q][t] = (owner && c < vcols && r < rows) ? P[(size_t)c * ld + r] : 0.f;
             }
+        // the columns are scaled (house.cuh)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const float sc = column_scale(warp_magnitude(x[q]), 0.f);
+            if (owner && lane == 0) back[2 * warp + q] = 1.f / sc;
+#pragma unroll
+            for (int t = 0; t < RPL; ++t) x[q][t] *= sc;
+        }
         if (warp == 0) {
 #pragma unroll
             for (int t = 0; t < RPL; ++t) pub[0][lane + 32 * t] = x[0][t];
@@ -313,7 +322,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (c >= vcols || r >= rows) continue;
                     P[(size_t)c * ld + r] = t == 0 && r < c ? 0.f : x[q][t];
                     if (t == 0 && R && r < vcols)
-                        R[b][(size_t)(j0 + c) * ldr + j0 + r] = r < c ? x[q][t] : (r == c ? diag[c] : 0.f);
+                        R[b][(size_t)(j0 + c) * ldr + j0 + r] =
+                            (r < c ? x[q][t] : (r == c ? diag[c] : 0.f)) * back[c];
                 }
             if (R) {
                 float* r_out = R[b];

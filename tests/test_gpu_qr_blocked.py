@@ -1,4 +1,5 @@
-"""GPU parity: blocked QRs whose copies in the workspace and whose Q differ in alignment."""
+"""GPU parity of the QRs with panels in registers: copies in the workspace and Q of different alignment, columns
+across the type's range."""
 import numpy as np
 import pytest
 
@@ -8,7 +9,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-def blocked_qr(mats, ldq=None):
+def run_qr(mats, ldq=None, blocked=True):
     """Q, R (64 bits) and info of a batch of matrices of one type; column j of Q starts on a multiple of ldq[b]
     elements after a 16-byte boundary."""
     import paper_1707_05141_gb300 as bs
@@ -26,8 +27,11 @@ def blocked_qr(mats, ldq=None):
     ta, tq, tr = (torch.from_numpy(x).cuda() for x in (fa, fq, fr))
     A, Q, R = bs.Batch.packed(ta, oa, m, n), bs.Batch.packed(tq, oq, m, n, ldq), bs.Batch.packed(tr, orr, n, n)
     info = torch.full((len(mats),), 7, dtype=torch.int32, device="cuda")
-    ws = torch.empty(bs.batched_qr_blocked_workspace(A), dtype=torch.uint8, device="cuda")
-    bs.batched_qr_blocked(A, Q, R, info, ws)
+    if blocked:
+        ws = torch.empty(bs.batched_qr_blocked_workspace(A), dtype=torch.uint8, device="cuda")
+        bs.batched_qr_blocked(A, Q, R, info, ws)
+    else:
+        bs.batched_qr(A, Q, R, info)
     torch.cuda.synchronize()
     hq, hr = tq.cpu().numpy().astype(np.float64), tr.cpu().numpy().astype(np.float64)
     q = [np.stack([hq[o + j * l:][:mm] for j in range(nn)], 1) for o, l, mm, nn in zip(oq, ldq, m, n)]
@@ -45,10 +49,43 @@ def test_aligned_q_beside_unaligned_workspace(dt, shapes):
     rng = np.random.default_rng(2)
     mats = [rng.standard_normal(s).astype(dt) for s in shapes]
     assert max(s[0] for s in shapes) * max(s[1] for s in shapes) % 2 == 1
-    q, r, info = blocked_qr(mats, [(s[0] + 3) // 4 * 4 for s in shapes])
+    q, r, info = run_qr(mats, [(s[0] + 3) // 4 * 4 for s in shapes])
     assert (info == 0).all()
     for a, qq, rr in zip(mats, q, r):
         a = a.astype(np.float64)
         assert np.abs(qq.T @ qq - np.eye(a.shape[1])).max() <= gate(dt), a.shape
         assert np.linalg.norm(a - qq @ rr) <= gate(dt) * np.linalg.norm(a), a.shape
         assert not np.tril(rr, -1).any()
+
+
+# the blocked one-CTA QR, and the blocked QR with one CTA, a cluster of two and one of four per panel
+@pytest.mark.parametrize("dt,m,n,blocked", [(np.float32, 200, 80, False), (np.float32, 300, 66, False),
+                                            (np.float32, 200, 80, True), (np.float32, 600, 40, True),
+                                            (np.float32, 2000, 64, True), (np.float64, 200, 40, True),
+                                            (np.float64, 1100, 33, True)])
+def test_columns_across_the_range(dt, m, n, blocked):
+    """Norms in the type's range are enough, also where the product of two columns' norms is not; dependent columns
+    (whose remainder after the first reflector is rounding) and independent ones."""
+    rng = np.random.default_rng(4)
+    a = rng.standard_normal((m, n))
+    big, small = (1e17, 1e-17) if dt == np.float32 else (1e150, 1e-150)
+    far = 1e5 if dt == np.float32 else 1e50
+    mats = []
+    for head, factor in ((big, far), (small, 1 / far)):
+        x = a.copy()
+        x[:, 0] *= head
+        x[:, 3] = x[:, 0] * factor   # a multiple of column 0
+        x[:, n - 1] = x[:, 0] / factor
+        mats.append(x.astype(dt))
+    mats += [(a * big).astype(dt), (a * small).astype(dt), (a * (small / 1e3)).astype(dt)]
+    x = a.copy()
+    x[:, 5] *= big
+    x[:, n - 2] *= small
+    mats.append(x.astype(dt))
+    q, r, info = run_qr(mats, blocked=blocked)
+    assert (info == 0).all()
+    for i, (x, qq, rr) in enumerate(zip(mats, q, r)):
+        x = x.astype(np.longdouble)
+        assert np.abs(qq.T @ qq - np.eye(n)).max() <= gate(dt), i
+        size = np.sqrt((x * x).sum(0))
+        assert (np.sqrt(((qq.astype(np.longdouble) @ rr.astype(np.longdouble) - x) ** 2).sum(0)) <= gate(dt) * size).all(), i
