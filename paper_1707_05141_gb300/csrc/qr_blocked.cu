@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
                 w[q] = j > c ? T(-2) * z : T(0);
                 if (j < c && rank == 0 && lane == 0) Gs[j][c] = z;
             }
-            if (rank == 0 && warp == 0 && lane == 0) rd[c] = alpha > T(0) ? -sa * back[c] : T(0);
+            if (rank == 0 && warp == 0 && lane == 0) rd[c] = alpha == T(0) ? T(0) : -sa * back[c];   // (a NaN stays one)
 #pragma unroll
             for (int t = 0; t < RPL; ++t) {
                 T v = pub[buf][lane + 32 * t] * inv;

@@ -89,3 +89,19 @@ def test_columns_across_the_range(dt, m, n, blocked):
         assert np.abs(qq.T @ qq - np.eye(n)).max() <= gate(dt), i
         size = np.sqrt((x * x).sum(0))
         assert (np.sqrt(((qq.astype(np.longdouble) @ rr.astype(np.longdouble) - x) ** 2).sum(0)) <= gate(dt) * size).all(), i
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("m", [100, 2000])
+def test_nan_stays_in_r(dt, m):
+    """No entry of R that a NaN reaches is a number, the diagonal included."""
+    rng = np.random.default_rng(6)
+    mats = [rng.standard_normal((m, n)).astype(dt) for n in (33, 1, 40)]
+    mats[0][m // 2, 32] = np.nan
+    mats[1][0, 0] = np.nan
+    mats[2][m - 1, 7] = np.nan
+    _, r, _ = run_qr(mats)
+    assert np.isnan(r[0][:, 32]).all() and np.isfinite(r[0][:, :32]).all()
+    assert np.isnan(r[1]).all()
+    assert np.isnan(r[2][:8, 7]).all()
+    assert np.isnan(np.diag(r[2])[7:]).all() and np.isfinite(r[2][:, :7]).all()
