@@ -13,7 +13,10 @@
 //   Q       the panels' block reflectors on [I; 0], last panel first, in place of V.
 // The order of the sums differs from qr_kernel's, so the randomized SVD, whose singular vectors move
 // with the last bit of R, keeps that one.
-// Measured (GB300, before -> here): 2000 matrices of 250 x 149 7.54 -> 3.62 ms, of 180 x 80 3.08 -> 1.64,
+// Their error does not grow: the products are summed in parts of 16 rows and an update's products by themselves before
+// they reach the column (Q of 250 x 149 Gaussian matrices against 64 bits: qr_kernel 4.06e-7, here 2.95e-7; 4.61e-7 with
+// one chain per thread through the products and through the column, for 2 % less time).
+// Measured (GB300, before -> here): 2000 matrices of 250 x 149 7.54 -> 3.69 ms, of 180 x 80 3.08 -> 1.64,
 // 20 of 250 x 149 0.54 -> 0.26.  One CTA per SM; by its code, the panels' chain of
 // barriers and the shared-memory loads of the updates bound it.
 #include <cuda_runtime.h>
@@ -127,20 +130,34 @@ __global__ void __launch_bounds__(kThreads, 1)
                     vp[x] = S + (size_t)(j0 + ti + 8 * x) * ld + j0;
                     cp[x] = S + (size_t)(c < n ? c : n - 1) * ld + j0;
                 }
-#pragma unroll 2
-                for (int r = g; r < rows4; r += groups) {
-                    Vec4 v[4], y[4];
+                // partial sums of 16 rows, then added: a single chain per thread (up to 128 rows) would err by more
+                // than the one-reflector form's 32 lanes and tree
+                for (int r0 = g; r0 < rows4; r0 += 4 * groups) {
+                    const int r1 = r0 + 4 * groups < rows4 ? r0 + 4 * groups : rows4;
+                    float part[4][4];
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        v[x] = ld4(vp[x] + 4 * r);
-                        y[x] = ld4(cp[x] + 4 * r);
+                    for (int x = 0; x < 4; ++x)
+#pragma unroll
+                        for (int z = 0; z < 4; ++z) part[x][z] = 0.f;
+#pragma unroll 2
+                    for (int r = r0; r < r1; r += groups) {
+                        Vec4 v[4], y[4];
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            v[x] = ld4(vp[x] + 4 * r);
+                            y[x] = ld4(cp[x] + 4 * r);
+                        }
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+#pragma unroll
+                            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                                for (int z = 0; z < 4; ++z) part[x][z] = fmaf(v[x].v[k], y[z].v[k], part[x][z]);
                     }
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
+                    for (int x = 0; x < 4; ++x)
 #pragma unroll
-                        for (int x = 0; x < 4; ++x)
-#pragma unroll
-                            for (int z = 0; z < 4; ++z) acc[x][z] = fmaf(v[x].v[k], y[z].v[k], acc[x][z]);
+                        for (int z = 0; z < 4; ++z) acc[x][z] += part[x][z];
                 }
             }
             for (int k = 0; k < groups; ++k) {   // the row groups, one after the other
@@ -180,16 +197,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                         make_float4(y[q][0], y[q][1], y[q][2], y[q][3]);
             }
             __syncthreads();
-            // C -= V Y: four rows, eight columns
+            // C -= V Y: four rows, eight columns; the product is summed by itself, so that C is rounded once per
+            // panel and not once per reflector
             const int units = rows4 * ((nc + 7) >> 3);
             for (int u = tid; u < units; u += kThreads) {
                 const int cg = u / rows4, r = j0 + 4 * (u - cg * rows4);
                 Vec4 o[8];
 #pragma unroll
-                for (int z = 0; z < 8; ++z) {
-                    const int c = cc + 8 * cg + z;
-                    o[z] = c < n ? ld4(S + (size_t)c * ld + r) : Vec4{};
-                }
+                for (int z = 0; z < 8; ++z) o[z] = Vec4{};
 #pragma unroll 4
                 for (int i = 0; i < kPw; ++i) {
                     const Vec4 v = ld4(S + (size_t)(j0 + i) * ld + r);
@@ -198,16 +213,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int z = 0; z < 4; ++z)
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            o[z].v[e] = fmaf(-v.v[e], y0.v[z], o[z].v[e]);
-                            o[z + 4].v[e] = fmaf(-v.v[e], y1.v[z], o[z + 4].v[e]);
+                            o[z].v[e] = fmaf(v.v[e], y0.v[z], o[z].v[e]);
+                            o[z + 4].v[e] = fmaf(v.v[e], y1.v[z], o[z + 4].v[e]);
                         }
                 }
 #pragma unroll
                 for (int z = 0; z < 8; ++z) {
                     const int c = cc + 8 * cg + z;
-                    if (c < n)
-                        *reinterpret_cast<float4*>(S + (size_t)c * ld + r) =
-                            make_float4(o[z].v[0], o[z].v[1], o[z].v[2], o[z].v[3]);
+                    if (c < n) {
+                        float* d = S + (size_t)c * ld + r;
+                        const Vec4 x = ld4(d);
+                        *reinterpret_cast<float4*>(d) = make_float4(x.v[0] - o[z].v[0], x.v[1] - o[z].v[1],
+                                                                    x.v[2] - o[z].v[2], x.v[3] - o[z].v[3]);
+                    }
                 }
             }
             __syncthreads();
