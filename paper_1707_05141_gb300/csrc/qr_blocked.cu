@@ -585,16 +585,21 @@ __global__ void __launch_bounds__(256) qb_panel_cluster_kernel(int p, int cs, un
 constexpr int kQwWarps = 16;                  // warps that own two panel columns each
 constexpr int kQwThreads = 32 * (kQwWarps + 1);   // and one that forms T
 
-// Panel p of matrix blockIdx.x / cs: CTA `rank` of its cluster holds panel rows [rank * 32 RPL, ...) in
-// registers, warp w the columns 2 w and 2 w + 1 (lane: rows lane + 32 t).  One reduction per column: the
+// Panel p of matrix blockIdx.x / cs: CTA `rank` of its cluster holds panel rows [rank * 32 RPL, ...) (FP64, whose
+// arithmetic bounds it: 32 rpl, the rows split evenly) in registers, warp w the columns 2 w and 2 w + 1 (lane: rows lane + 32 t).  One reduction per column: the
 // raw pivot x (zero above row c) is multiplied with all 32 columns at once, since with v = (x + sg alpha
 // e_c) inv the products v^T x_j (the update of column j > c) and v_j^T v (the entry of V^T V for T, j < c)
 // are inv (x^T x_j + sg alpha x_j(c)); norm, updates and T come from the same 32 sums.  They are pushed to
 // every CTA of the cluster (distributed shared memory), so a column costs one cluster barrier and one CTA
 // barrier.  Bound by that latency.  A 2000-row panel (8 matrices, 4-CTA clusters of 500 rows) took 245 us
 // with the panel in shared memory, two cluster barriers and three passes per column; it takes 53 us here.
-template <typename T, int RPL>
-__global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, unsigned char* ws, QbLayout L, QbInts I)
+// FP64 is bound by its arithmetic (an FP64 instruction of a warp takes 16 cycles of an SM): one warp forms the
+// reflector, two columns share a butterfly, rows past the end and finished columns are not multiplied.  500
+// matrices of 200 x 64 with their Q took 3.47 ms with the panels in shared memory, 5.40 ms with every warp forming the
+// reflector, and take 3.18 ms; 8 of 512 x 64 1.81, 1.41 and 0.95 ms.
+template <typename T, int RPL, int MINB>
+__global__ void __launch_bounds__(kQwThreads, MINB) qw_panel_kernel(int p, int cs, int rpl, unsigned char* ws, QbLayout L,
+                                                                 QbInts I)
 {
     __shared__ T pub[2][RPL * 32];            // the pivot column of this CTA's rows
     __shared__ T xch[2][kClusterMax][kPw];    // the CTAs' partial products with the pivot
@@ -608,11 +613,14 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
     const int mm = I.mm[b], nn = I.nn[b];
     const int j0 = p * kPw;
     if (j0 >= nn) return;                     // the whole cluster (one matrix) leaves together
-    const int rows = mm - j0, r0 = rank * 32 * RPL;
-    const int nr = rows - r0 < 0 ? 0 : (rows - r0 > 32 * RPL ? 32 * RPL : rows - r0);
+    const int rows = mm - j0, slab = 32 * (sizeof(T) == 8 ? rpl : RPL), r0 = rank * slab;
+    const int nr = rows - r0 < 0 ? 0 : (rows - r0 > slab ? slab : rows - r0);
     const int vcols = nn - j0 < kPw ? nn - j0 : kPw;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool owner = warp < kQwWarps;
+    const bool owner = warp < kQwWarps, busy = 2 * warp < vcols;   // (vcols <= 2 kQwWarps)
+    constexpr bool F64 = sizeof(T) == 8;
+    __shared__ T scal[2];                     // FP64: sign(x0) alpha and 1 / ||v|| of the column
+    auto row_block = [&](int t) { return !F64 || 32 * t < nr; };   // FP64: rows past the end are not multiplied
     T* X = qb_X<T>(ws, L, b) + (size_t)j0 * mm + j0 + r0;   // panel element (row r0, column 0)
     T x[2][RPL];
 #pragma unroll
@@ -624,19 +632,19 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
         }
     // the columns scaled (house.cuh) by their largest magnitude in all of the cluster's rows
     unsigned mag[2] = {0, 0};
-    if (owner) {
+    if (busy) {
         mag[0] = warp_magnitude(x[0]);
         mag[1] = warp_magnitude(x[1]);
     }
     if (cs > 1) {
         cluster.sync();                       // every CTA of the cluster runs before the first push
-        if (owner && lane < cs) {
+        if (busy && lane < cs) {
             unsigned* g = cluster.map_shared_rank(&mags[rank][2 * warp], lane);
             g[0] = mag[0];
             g[1] = mag[1];
         }
         cluster.sync();
-        if (owner)
+        if (busy)
             for (int k = 0; k < cs; ++k) {
                 mag[0] = max(mag[0], mags[k][2 * warp]);
                 mag[1] = max(mag[1], mags[k][2 * warp + 1]);
@@ -664,18 +672,30 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
     __syncthreads();
     for (int c = 0; c < vcols; ++c) {
         const int buf = c & 1;
-        if (owner) {
+        if (busy) {
             T s[2] = {T(0), T(0)};
 #pragma unroll
             for (int t = 0; t < RPL; ++t) {
+                if (!row_block(t)) break;
                 const T v = pub[buf][lane + 32 * t];
                 s[0] = fma(v, x[0][t], s[0]);
                 s[1] = fma(v, x[1][t], s[1]);
             }
+            if constexpr (F64) {
+                // both columns in one butterfly, half of the lanes each after its first level: the same sums by half
+                // of the additions
+                const T other = __shfl_xor_sync(0xffffffffu, lane < 16 ? s[1] : s[0], 16);
+                T h = (lane < 16 ? s[0] : s[1]) + other;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
-                s[1] += __shfl_xor_sync(0xffffffffu, s[1], o);
+                for (int o = 8; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+                s[0] = __shfl_sync(0xffffffffu, h, 0);
+                s[1] = __shfl_sync(0xffffffffu, h, 16);
+            } else {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+                    s[1] += __shfl_xor_sync(0xffffffffu, s[1], o);
+                }
             }
             const T e0 = __shfl_sync(0xffffffffu, x[0][0], c), e1 = __shfl_sync(0xffffffffu, x[1][0], c);
             if (lane < cs) {
@@ -692,13 +712,61 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
                     pr[1] = e1;
                 }
             }
-        } else if (rank == 0 && c > 0) {
+        } else if (!owner && rank == 0 && c > 0) {
             t_column(c - 1);
             __syncwarp();
         }
         if (cs > 1) cluster.sync();
         else __syncthreads();
-        if (owner) {
+        if constexpr (F64) {
+            // by one warp, in place of the pivot: a square root and a reciprocal one are about a hundred FP64
+            // instructions of 16 cycles on an SM; by all 16 warps they took longer than the products
+            if (c >> 1 == warp) {
+                T tot = T(0);
+                for (int k = 0; k < cs; ++k) tot += xch[buf][k][c];
+                const T x0 = row[buf][c];
+                const T alpha = dsqrt(tot);
+                const T sa = x0 >= T(0) ? alpha : -alpha;   // sign(x0) alpha
+                const T inv = alpha > T(0) ? drsqrt(T(2) * alpha * (alpha + dabs(x0))) : T(0);
+                const T vc = (x0 + sa) * inv;               // v's entry in row c
+                if (lane == 0) {
+                    scal[0] = sa;
+                    scal[1] = inv;
+                    if (rank == 0) rd[c] = alpha == T(0) ? T(0) : -sa * back[c];   // (a NaN stays one)
+                }
+#pragma unroll
+                for (int t = 0; t < RPL; ++t) {
+                    if (!row_block(t)) break;
+                    T v = pub[buf][lane + 32 * t] * inv;
+                    if (t == 0 && rank == 0 && lane == c) v = vc;
+                    pub[buf][lane + 32 * t] = v;
+                    if (!(t == 0 && rank == 0 && lane < c)) {   // column c becomes v
+                        if (c & 1) x[1][t] = v;
+                        else x[0][t] = v;
+                    }
+                }
+            }
+            __syncthreads();
+            if (busy) {
+                // half of the lanes form the factor of each column
+                const int j = 2 * warp + (lane >> 4);
+                T sj = T(0);
+                for (int k = 0; k < cs; ++k) sj += xch[buf][k][j];
+                const T z = scal[1] * fma(scal[0], row[buf][j], sj);
+                if (j < c && rank == 0 && (lane & 15) == 0) Gs[j][c] = z;
+                if (2 * warp + 1 > c) {
+                    const T w = j > c ? T(-2) * z : T(0);
+                    const T w0 = __shfl_sync(0xffffffffu, w, 0), w1 = __shfl_sync(0xffffffffu, w, 16);
+#pragma unroll
+                    for (int t = 0; t < RPL; ++t) {
+                        if (!row_block(t)) break;
+                        const T v = pub[buf][lane + 32 * t];
+                        if (2 * warp > c) x[0][t] = fma(w0, v, x[0][t]);
+                        x[1][t] = fma(w1, v, x[1][t]);
+                    }
+                }
+            }
+        } else if (busy) {
             T tot = T(0), s[2] = {T(0), T(0)};
             for (int k = 0; k < cs; ++k) {
                 tot += xch[buf][k][c];
@@ -719,23 +787,25 @@ __global__ void __launch_bounds__(kQwThreads, 1) qw_panel_kernel(int p, int cs, 
                 if (j < c && rank == 0 && lane == 0) Gs[j][c] = z;
             }
             if (rank == 0 && warp == 0 && lane == 0) rd[c] = alpha == T(0) ? T(0) : -sa * back[c];   // (a NaN stays one)
-#pragma unroll
-            for (int t = 0; t < RPL; ++t) {
-                T v = pub[buf][lane + 32 * t] * inv;
-                if (t == 0 && rank == 0 && lane == c) v = vc;
-                x[0][t] = fma(w[0], v, x[0][t]);
-                x[1][t] = fma(w[1], v, x[1][t]);
-                if (c >> 1 == warp && !(t == 0 && rank == 0 && lane < c)) {   // column c becomes v
-                    if (c & 1) x[1][t] = v;
-                    else x[0][t] = v;
-                }
-            }
-            if ((c + 1) >> 1 == warp && c + 1 < vcols) {   // publish the next pivot, zero above its row
+            if (2 * warp + 1 >= c) {   // (the columns of the other warps are finished)
 #pragma unroll
                 for (int t = 0; t < RPL; ++t) {
-                    const T y = (c + 1) & 1 ? x[1][t] : x[0][t];
-                    pub[buf ^ 1][lane + 32 * t] = t == 0 && rank == 0 && lane <= c ? T(0) : y;
+                    T v = pub[buf][lane + 32 * t] * inv;
+                    if (t == 0 && rank == 0 && lane == c) v = vc;
+                    x[0][t] = fma(w[0], v, x[0][t]);
+                    x[1][t] = fma(w[1], v, x[1][t]);
+                    if (c >> 1 == warp && !(t == 0 && rank == 0 && lane < c)) {   // column c becomes v
+                        if (c & 1) x[1][t] = v;
+                        else x[0][t] = v;
+                    }
                 }
+            }
+        }
+        if (busy && (c + 1) >> 1 == warp && c + 1 < vcols) {   // publish the next pivot, zero above its row
+#pragma unroll
+            for (int t = 0; t < RPL; ++t) {
+                const T y = (c + 1) & 1 ? x[1][t] : x[0][t];
+                pub[buf ^ 1][lane + 32 * t] = t == 0 && rank == 0 && lane <= c ? T(0) : y;
             }
         }
         __syncthreads();
@@ -867,12 +937,17 @@ __global__ void __launch_bounds__(256, 3) qw_apply_kernel(int p, int trans, int 
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[a][c] = T(0);
+    // FP64, whose arithmetic bounds it: rows past the end and column blocks past the last one are not multiplied, nor
+    // T's zero triangle
+    constexpr bool F64 = sizeof(T) == 8;
+    const int ablk = F64 ? (vcols + 7) >> 3 : 4, cblk = F64 ? (ncol + 7) >> 3 : 4;
     for (int s = rank; s < slabs; s += cs) {
         __syncthreads();
         stage(s);
         __syncthreads();
+        const int r1 = F64 && rows - s * SR < (g + 1) * (SR / 4) ? rows - s * SR : (g + 1) * (SR / 4);
 #pragma unroll 2
-        for (int r = g * (SR / 4); r < (g + 1) * (SR / 4); r += VE) {
+        for (int r = g * (SR / 4); r < r1; r += VE) {
             T v[4][VE], x[4][VE];
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
@@ -882,9 +957,14 @@ __global__ void __launch_bounds__(256, 3) qw_apply_kernel(int p, int trans, int 
 #pragma unroll
             for (int k = 0; k < VE; ++k)
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
+                for (int a = 0; a < 4; ++a) {
+                    if (F64 && a >= ablk) break;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[a][c] = fma(v[a][k], x[c][k], acc[a][c]);
+                    for (int c = 0; c < 4; ++c) {
+                        if (F64 && c >= cblk) break;
+                        acc[a][c] = fma(v[a][k], x[c][k], acc[a][c]);
+                    }
+                }
         }
     }
     // the four row groups, one after the other, into Wp
@@ -931,8 +1011,9 @@ __global__ void __launch_bounds__(256, 3) qw_apply_kernel(int p, int trans, int 
         // Y = op(T) W, thread: row i, four columns
         const int i = tid >> 3, c = (tid & 7) * 4;
         T y[4] = {T(0), T(0), T(0), T(0)};
+        const int k0 = F64 && !trans ? i & ~3 : 0, k1 = F64 && trans ? (i | 3) + 1 : kPw;   // (a warp's four rows)
 #pragma unroll 8
-        for (int k = 0; k < kPw; ++k) {
+        for (int k = k0; k < k1; ++k) {
             const T tk = Tsm[k * LW + i];
 #pragma unroll
             for (int q = 0; q < 4; ++q) y[q] = fma(tk, Ws[k * LW + c + q], y[q]);
@@ -954,6 +1035,7 @@ __global__ void __launch_bounds__(256, 3) qw_apply_kernel(int p, int trans, int 
             __syncthreads();
         }
         const int r = rg * VE, gr = s * SR + r;
+        if (F64 && (gr >= rows || cg0 >= ncol)) continue;   // (no barrier is left out: all threads make the same passes)
         T o[NC][VE];
 #pragma unroll
         for (int j = 0; j < NC; ++j) qw_load(Cs + (cg0 + j) * LD + r, o[j]);
@@ -1156,14 +1238,18 @@ static int qw_launch_panel(int p, int batch, int rows, unsigned char* ws, const 
     int cs = (rows + 511) / 512;
     if (cs > kClusterMax) cs = kClusterMax;
     const int rpl = ((rows + cs - 1) / cs + 31) / 32;
-    void (*kern)(int, int, unsigned char*, QbLayout, QbInts);
-    if (rpl <= 4) kern = qw_panel_kernel<T, 4>;
-    else if (rpl <= 8) kern = qw_panel_kernel<T, 8>;
-    else if (rpl <= 16) kern = qw_panel_kernel<T, 16>;
-    else if (rpl <= 24) kern = qw_panel_kernel<T, 24>;
-    else if (sizeof(T) == 4 && rpl <= 48) kern = qw_panel_kernel<T, sizeof(T) == 4 ? 48 : 24>;
+    void (*kern)(int, int, int, unsigned char*, QbLayout, QbInts);
+    // more matrices than SMs: two CTAs per SM, with 56 registers a thread (500 of 256 x 100 0.82 -> 0.73 ms; fewer matrices
+    // run faster with more: 8 of 256 x 100 0.187 against 0.212 ms)
+    const bool many = batch > 152;
+    if (rpl <= 2) kern = qw_panel_kernel<T, 2, 2>;
+    else if (rpl <= 4) kern = many ? qw_panel_kernel<T, 4, 2> : qw_panel_kernel<T, 4, 1>;
+    else if (rpl <= 8) kern = many ? qw_panel_kernel<T, 8, 2> : qw_panel_kernel<T, 8, 1>;
+    else if (rpl <= 16) kern = qw_panel_kernel<T, 16, 1>;
+    else if (rpl <= 24) kern = qw_panel_kernel<T, 24, 1>;
+    else if (sizeof(T) == 4 && rpl <= 48) kern = qw_panel_kernel<T, sizeof(T) == 4 ? 48 : 24, 1>;
     else return BSVD_ERR_UNSUPPORTED;
-    return qw_launch(kern, batch * cs, kQwThreads, 0, cs, st, p, cs, ws, L, I);
+    return qw_launch(kern, batch * cs, kQwThreads, 0, cs, st, p, cs, rpl, ws, L, I);
 }
 
 // CTAs per tile of the block reflector: enough slabs of rows to fill the GPU, at most the slabs there are

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int j0 = 0; j0 < n; j0 += kPw) {
         const int vcols = n - j0 < kPw ? n - j0 : kPw, rows = m - j0;
         float* P = S + (size_t)j0 * ld + j0;
-        const bool owner = warp < kWarps;
+        const bool owner = warp < kWarps, busy = 2 * warp < vcols;   // (vcols <= 2 kWarps)
         float x[2][RPL];
 #pragma unroll
         for (int q = 0; q < 2; ++q)
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncthreads();
         for (int c = 0; c < vcols; ++c) {
             const int buf = c & 1;
-            if (owner) {
+            if (busy) {
                 float s0 = 0.f, s1 = 0.f;
 #pragma unroll
                 for (int t = 0; t < RPL; ++t) {
@@ -287,12 +287,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     row[buf][2 * warp] = e0;
                     row[buf][2 * warp + 1] = e1;
                 }
-            } else if (c > 0) {
+            } else if (!owner && c > 0) {
                 t_column(c - 1);
                 __syncwarp();
             }
             __syncthreads();
-            if (owner) {
+            if (busy) {
                 const float tot = sum[buf][c], x0 = row[buf][c];
                 const float alpha = dsqrt(tot);
                 const float sa = x0 >= 0.f ? alpha : -alpha;   // sign(x0) alpha
@@ -308,15 +308,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (j < c && lane == 0) Gs[j][c] = z;
                 }
                 if (tid == 0) diag[c] = alpha > 0.f ? -sa : 0.f;
+                if (2 * warp + 1 >= c) {   // (the columns of the other warps are finished)
 #pragma unroll
-                for (int t = 0; t < RPL; ++t) {
-                    float v = pub[buf][lane + 32 * t] * inv;
-                    if (t == 0 && lane == c) v = vc;
-                    x[0][t] = fmaf(w[0], v, x[0][t]);
-                    x[1][t] = fmaf(w[1], v, x[1][t]);
-                    if (c >> 1 == warp && !(t == 0 && lane < c)) {   // column c becomes v
-                        if (c & 1) x[1][t] = v;
-                        else x[0][t] = v;
+                    for (int t = 0; t < RPL; ++t) {
+                        float v = pub[buf][lane + 32 * t] * inv;
+                        if (t == 0 && lane == c) v = vc;
+                        x[0][t] = fmaf(w[0], v, x[0][t]);
+                        x[1][t] = fmaf(w[1], v, x[1][t]);
+                        if (c >> 1 == warp && !(t == 0 && lane < c)) {   // column c becomes v
+                            if (c & 1) x[1][t] = v;
+                            else x[0][t] = v;
+                        }
                     }
                 }
                 if ((c + 1) >> 1 == warp && c + 1 < vcols) {   // publish the next pivot
@@ -409,7 +411,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Which bounds take this kernel.  It holds an SM alone, so it loses to qr_kernel, several CTAs of which share
 // one, where a matrix is small (2000 matrices, before / here: 100 x 70 1.19 / 1.33 ms, 128 x 70 1.22 /
 // 1.36, 256 x 64 1.11 / 1.19, 300 x 34 0.78 / 0.97), and wins beyond (160 x 70 2.50 / 1.47, 200 x 66 2.35
-// / 1.47, 300 x 66 3.82 / 1.87, 257 x 64 2.18 / 1.46, 500 x 40 1.99 / 1.18).  Matrices that are nearly square
+// / 1.47, 300 x 66 3.82 / 1.87, 257 x 64 2.18 / 1.46, 500 x 40 1.99 / 1.18).  At the line, 48 to 51 columns, it
+// loses where R alone is wanted of thousands (2000 of 300 x 50 0.84 / 0.89 ms; with Q 1.46 / 1.21, 20 of them 0.144
+// / 0.064): both calls give the same R, so both take it.  Matrices that are nearly square
 // keep qr_kernel's order of sums: the last column of Q of a random square matrix is determined only
 // to the size of R(n, n), which over a batch comes close to zero.
 int launch_qr_wy(int batch, int max_m, int max_n, void* const* A, const int* M, const int* N, const int* LDA,

@@ -1,5 +1,5 @@
 """GPU parity of the QRs with panels in registers: copies in the workspace and Q of different alignment, columns
-across the type's range."""
+across the type's range, more matrices than SMs."""
 import numpy as np
 import pytest
 
@@ -105,3 +105,20 @@ def test_nan_stays_in_r(dt, m):
     assert np.isnan(r[1]).all()
     assert np.isnan(r[2][:8, 7]).all()
     assert np.isnan(np.diag(r[2])[7:]).all() and np.isfinite(r[2][:, :7]).all()
+
+
+# more matrices than SMs take the panels with half of the registers a thread; 32, 64, 128 and 256 rows are their sizes
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("rows", [[33, 40, 64], [65, 66, 128], [129, 200, 256], [257, 300, 288]])
+def test_more_matrices_than_sms(dt, rows):
+    rng = np.random.default_rng(rows[0])
+    shapes = [(rows[i % 3], n) for i, n in enumerate(rng.integers(1, 38, 165))]
+    mats = [rng.standard_normal((m, min(m, n))).astype(dt) for m, n in shapes]
+    mats[7][:, 0] = 0
+    q, r, info = run_qr(mats)
+    assert (info == 0).all()
+    for b, (a, qq, rr) in enumerate(zip(mats, q, r)):
+        a = a.astype(np.float64)
+        assert np.abs(qq.T @ qq - np.eye(a.shape[1])).max() <= gate(dt), (b, a.shape)
+        assert np.linalg.norm(a - qq @ rr) <= gate(dt) * np.linalg.norm(a), (b, a.shape)
+        assert not np.tril(rr, -1).any()
