@@ -60,7 +60,7 @@ struct Red3 {
 // MINB is the number of matrices (CTAs) the launch bound asks to keep resident per SM; it caps
 // the register allocation at 65536 / (NS * PARTS * MINB), trading scheduling freedom against
 // occupancy.  Several values are instantiated and the autotuner picks one per size bin.
-template <typename T, int NS, int PARTS, int RA, int RV, int MINB, bool FAST, bool PRE, bool P64, bool CARRY>
+template <typename T, int NS, int PARTS, int RA, int RV, int MINB, bool FAST, bool PRE, bool P64, bool CARRY, bool RN>
 __global__ void __launch_bounds__(NS * PARTS, MINB)
     jacobi_reg_kernel(int batch, T* const* A, const int* M, const int* N, const int* LDA, T* const* Sout, T* const* U,
                       const int* LDU, T* const* V, const int* LDV, double tol_in, int max_sweeps, int* info,
@@ -74,12 +74,11 @@ __global__ void __launch_bounds__(NS * PARTS, MINB)
     // rotation parameters (zeta, t, c, s) and the rotation test in the working precision, or in
     // FP64 for FP32 data (P64): the Gram entries are summed in T, then promoted
     typedef typename std::conditional<P64, double, T>::type P;
-    // carried norms leave one sum per step, and the chain of the parameters behind it shows: branch-free
-    // ones (rnmath.cuh) and no parameters in a step that rotates nothing: 500 / 10 000 preconditioned 32 x 32
-    // matrices 0.208 / 1.30 -> 0.189 / 1.24 ms.
-    // Where all three sums are formed, they hide the chain and the built-in operations' fewer
-    // instructions are 2 to 9 % faster.
-    constexpr bool RN = CARRY && !P64 && sizeof(T) == 4;
+    // RN: branch-free parameters (rnmath.cuh), and none in a step that rotates nothing.  Carried norms leave one sum
+    // per step, and the chain of the parameters behind it shows: 500 / 10 000 preconditioned 32 x 32 matrices
+    // 0.208 / 1.30 -> 0.189 / 1.24 ms.  Where all three sums are formed, they hide the chain and the
+    // built-in operations' fewer instructions are 2 to 9 % faster.
+    static_assert(!RN || (CARRY && !P64 && sizeof(T) == 4), "FP32 parameters from one sum");
 
     __shared__ Red3<T> red[2][NW > 1 ? NW : 1][32];
     __shared__ T sig_s[NC];
@@ -590,43 +589,61 @@ __global__ void __launch_bounds__(NS * PARTS, MINB)
     }
 }
 
-// The plain 32-slot FP32 variants have both forms: the one above (two or four warps with half or a quarter
-// of the rows of W and V each) and jacobi_wv.cu's (half as many W warps with all the columns in half the
-// lanes, V elsewhere).  Up to two matrices per SM a step's latency is what counts, and it is shorter
-// above: 54 x 45, 16 / 304 matrices with U and V 0.80 / 0.84 ms against 0.86 / 0.95.  Beyond, the issue
-// slots count: 608 matrices 1.05 against 1.02 ms, 8000 10.9 against 9.6 (120 x 50: 1.39 against 0.96 and
-// 17.4 against 11.6).  Without U and V two parts have nothing to keep out of W's warps: 0.83 against 0.88 ms
-// at 608, 8.25 against 8.22 at 8000.  (Preconditioned or with FP64 parameters, jacobi_wv.cu is faster
-// from 16 matrices on.)
-static bool use_wv(int parts, bool vectors, int batch)
+// The 32-slot FP32 variants that are not preconditioned have both forms: the one above (two or four warps with half
+// or a quarter of the rows of W and V each) and jacobi_wv.cu's (half as many W warps with all the columns in half
+// the lanes, V elsewhere).  While the matrices fit the SMs at once a step's latency is what counts, and it is
+// shorter above; beyond, the issue slots count.  Time above / time there with U and V, by matrices per SM (the
+// third column: one matrix more than two; the fifth: one more than four):
+//                                       0.1    2     2+    3    4+    14
+//   three sums, 64 x 64                             0.96  1.01  1.09  1.11
+//   three sums, 54 x 45                 0.93  0.88  1.00  1.00  1.03  1.06
+//   ... with 4 CTAs per SM                          0.96  0.96  1.30  1.17
+//   carried norms, 64 x 64                          1.02  1.09  1.16  1.14
+//   carried norms, 48 x 48                          0.91  0.94  1.06  1.04
+//   FP64 parameters, 54 x 45            0.96  1.00  1.21  1.25  1.70  1.89
+//   four parts, 128 x 64                            1.38  1.49  1.24  1.42
+// Without U and V two parts with FP32 parameters have nothing to keep out of W's warps: 1.00 at most.
+// Preconditioned, jacobi_wv.cu is faster from one matrix on.
+static bool use_wv(int parts, int minb, bool p64, bool carry, int nn, bool vectors, int batch)
 {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return batch > 2 * sms && (parts == 4 || vectors);
+    if (parts == 4 || p64) return batch > 2 * sms;
+    const int per = carry ? (nn > 60 ? 2 : 4) : (minb == 4 ? 4 : 3);
+    return vectors && batch > per * sms;
 }
 
 template <typename T, int NS, int PARTS, int RA, int RV, int MINB, bool FAST, bool PRE, bool P64, bool CARRY>
-static int launch_reg(int batch, void* const* A, const int* M, const int* N, const int* LDA, void* const* S,
+static int launch_reg(int nn, int batch, void* const* A, const int* M, const int* N, const int* LDA, void* const* S,
                       void* const* U, const int* LDU, void* const* V, const int* LDV, double tol, int max_sweeps,
                       int* info, long long* rot, cudaStream_t st, ItemList wl)
 {
-    if constexpr (sizeof(T) == 4 && NS == 32 && RA == 32 && FAST) {
+    constexpr bool wv = sizeof(T) == 4 && NS == 32 && RA == 32 && FAST;
+    if constexpr (wv) {
         // 32 slots, parts of 32 rows: W and V in separate warps (jacobi_wv.cu; the same sums and
         // rotations, bit for bit: 20 000 preconditioned 64 x 64 matrices 18.6 -> 13.8 ms).  A W warp there
         // has twice the columns and half the steps' barriers of a warp here, so its step takes longer
         // and more matrices fit an SM.
-        if (PRE || P64 || use_wv(PARTS, U || V, batch))
+        if (PRE || use_wv(PARTS, MINB, P64, CARRY, nn, U || V, batch))
             return launch_jacobi_wv(PARTS == 4, PRE, P64, CARRY, batch, A, M, N, LDA, S, U, LDU, V, LDV, tol,
                                     max_sweeps, info, rot, st, wl);
     }
-    if constexpr (!(sizeof(T) == 4 && NS == 32 && RA == 32 && FAST && (PRE || P64))) {
-        auto kern = jacobi_reg_kernel<T, NS, PARTS, RA, RV, MINB, FAST, PRE, P64 && sizeof(T) == 4, CARRY>;
-        const int grid = item_grid(kern, NS * PARTS, 0, wl, batch, st);
-        if (grid == 0) return BSVD_ERR_CUDA;
-        kern<<<grid, NS * PARTS, 0, st>>>(batch, (T* const*)A, M, N, LDA, (T* const*)S, (T* const*)U, LDU,
-                                          (T* const*)V, LDV, tol, max_sweeps, info, rot, wl);
-        return cudaGetLastError() == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
+    if constexpr (!(wv && PRE)) {
+        auto launch = [&](auto kern) {
+            const int grid = item_grid(kern, NS * PARTS, 0, wl, batch, st);
+            if (grid == 0) return BSVD_ERR_CUDA;
+            kern<<<grid, NS * PARTS, 0, st>>>(batch, (T* const*)A, M, N, LDA, (T* const*)S, (T* const*)U, LDU,
+                                              (T* const*)V, LDV, tol, max_sweeps, info, rot, wl);
+            return cudaGetLastError() == cudaSuccess ? BSVD_SUCCESS : BSVD_ERR_CUDA;
+        };
+        // the branch-free parameters: carried norms of preconditioned or full-width matrices (16 plain 64 x 64 ones
+        // 6 % faster, of 56 x 56 3 % and 54 x 45 4 % slower)
+        if constexpr (CARRY && !P64 && sizeof(T) == 4) {
+            if (PRE || nn > 60) return launch(jacobi_reg_kernel<T, NS, PARTS, RA, RV, MINB, FAST, PRE, false, true, true>);
+        }
+        if constexpr (!(CARRY && PRE && sizeof(T) == 4))
+            return launch(jacobi_reg_kernel<T, NS, PARTS, RA, RV, MINB, FAST, PRE, P64, CARRY, false>);
     }
     return BSVD_ERR_UNSUPPORTED;  // (not reached)
 }
@@ -682,7 +699,7 @@ int launch_jacobi_reg(int batch, int max_m, int max_n, int variant, void* const*
         ++seen;                                                                                             \
         if (variant == 0 || variant == seen)                                                                \
             return launch_reg<T, NS_, PARTS_, RA_, RV_, MINB_, FAST_, PRE_, P64_, CARRY_>(                        \
-                batch, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps, info, rot, st, wl);                      \
+                nn, batch, A, M, N, LDA, S, U, LDU, V, LDV, tol, max_sweeps, info, rot, st, wl);                      \
     }
     if constexpr (sizeof(T) == 4) {
         BSVD_REG_VARIANTS_F32(BSVD_TRY)
