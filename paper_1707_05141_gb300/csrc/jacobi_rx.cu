@@ -101,7 +101,9 @@ __device__ __forceinline__ bool rx_rotation(float al, float be, float ga, P tol,
         t = zeta >= 0.f ? t : -t;
         const float cf = rn_rsqrt12(fmaf(t, t, 1.f));
         auto in = [](float x) { return x >= 0x1p-100f && x <= 0x1p100f; };
-        // (the test itself needs the norms' range, the parameters the rest)
+        // (the test itself needs the norms' range, the parameters the rest; zeta, 0 or at least 2^-26 since d is a
+        // multiple of a last place and |ga| at most the norms, is then a quotient in range, and its square plus 1
+        // below 2^118)
         const bool safe = in(al) && in(be) && (!rot || (in(fabsf(g2)) && (d == 0.f || in(fabsf(d))) && az < 0x1p59f));
         if (__any_sync(kRxFull, pos && !safe)) {
             float cs[2];
@@ -438,7 +440,6 @@ __global__ void __launch_bounds__(kRx8Cols / 2 * kRx8Lanes)
     float* xv = xw + 2 * nslot_max * kRx8LdW;                    // [2][nslot_max][kRx8LdV]
     int* xc = reinterpret_cast<int*>(xv + 2 * nslot_max * kRx8LdV);   // [2][nslot_max] column ids
     float* sig = reinterpret_cast<float*>(xc + 2 * nslot_max);   // [max_np] singular values by column id
-    int* rank = reinterpret_cast<int*>(sig + max_np);            // [max_np]
     const int tid = threadIdx.x;
     const int s = tid / G, g = tid % G;
 
@@ -463,7 +464,6 @@ __global__ void __launch_bounds__(kRx8Cols / 2 * kRx8Lanes)
             }
             continue;
         }
-        const bool accV = tr ? wantU : wantV;
         const bool live = s < ns, wrap = s == ns - 1;
         int colL = 2 * s, colR = 2 * s + 1;
         const float* a = A[b];
@@ -634,7 +634,7 @@ static int launch_rx8(int batch, int max_mm, int max_np, void* const* A, const i
 {
     auto kern = jacobi_rx8_kernel;
     const int ns = max_np / 2;
-    const size_t smem = sizeof(float) * (2 * ns * (kRx8LdW + kRx8LdV) + 2 * ns + 2 * max_np);
+    const size_t smem = sizeof(float) * (2 * ns * (kRx8LdW + kRx8LdV) + 2 * ns + max_np);
     const int threads = (ns * kRx8Lanes + 31) & ~31;
     const int grid = item_grid(kern, threads, smem, wl, batch, st);
     if (grid == 0) return BSVD_ERR_CUDA;
