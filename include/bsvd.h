@@ -75,6 +75,7 @@ extern "C" {
  * Q and R are therefore unique; a zero column gives the identity reflector.
  * Limits: max_m <= 1024 and max_m * max_n * sizeof(element) <= 200 KiB (the matrix is factored
  * in shared memory); otherwise BSVD_ERR_UNSUPPORTED.
+ * Which kernel runs follows from the type and the bounds; last bits may differ between bounds.
  */
 int batched_qr(int dtype, int batch, int max_m, int max_n,
                void* const* dA, const int* d_m, const int* d_n, const int* d_lda,
@@ -92,20 +93,21 @@ size_t batched_qr_blocked_workspace(int dtype, int batch, int max_m, int max_n);
  * batched_qr_blocked -- the same reduced Householder QR (Algorithm 1, same reflectors and signs) for
  * matrices beyond batched_qr's shared-memory kernel: the blocked factorisation Section 3.1 leaves to
  * larger matrices and Section 3.2 names for large squares.  Each matrix is copied to the workspace
- * and factored in 32-column panels: the panel (all rows below its first) is factored on chip, its
+ * and factored in 32-column panels: the panel (all rows below its first) is factored in registers, its
  * reflectors are gathered in the compact WY form H_j ... H_{j+31} = I - V T V^T, and the trailing
- * columns are updated as C - V T^T (V^T C), streamed through shared memory in 128-row chunks.
+ * columns are updated as C - V T^T (V^T C), in slabs of 256 rows (FP64: 128) in shared memory that a
+ * thread-block cluster splits where the batch leaves SMs idle.
  * Q = H_0 ... H_{n-1} [I; 0] is formed by applying the panels' block reflectors, last panel first.
- * A panel taller than one CTA's shared memory holds (1533 rows FP32, 733 FP64) is factored by a
- * thread-block cluster of up to 8 CTAs, each with a slab of its rows in shared memory; the
- * reflectors' norms and products are summed across the cluster through distributed shared memory.
+ * A panel of more than 512 rows is factored by a thread-block cluster of up to 8 CTAs, each with a
+ * slab of its rows; a column's products with the panel are summed across the cluster through
+ * distributed shared memory (one cluster barrier and one CTA barrier per column).
  *
  *   Arguments as batched_qr, plus:
  *   workspace  DEVICE buffer of at least batched_qr_blocked_workspace(...) bytes, caller-owned,
  *              contents need not be initialised; not used after the stream work completes.
  *              Smaller -> BSVD_ERR_WORKSPACE.
- * Limits: max_m <= batched_qr_blocked_max_rows(dtype) (8 slabs of a 32-column panel, each in
- * 200 KiB of one CTA's shared memory: 11976 rows FP32, 5576 FP64); any max_n <= max_m.  Otherwise
+ * Limits: max_m <= batched_qr_blocked_max_rows(dtype) (11976 rows FP32, 5576 FP64: what the block
+ * tier's panels, 8 slabs in 200 KiB of shared memory each, take too); any max_n <= max_m.  Otherwise
  * BSVD_ERR_UNSUPPORTED.  d_info[b] as batched_qr.
  */
 int batched_qr_blocked(int dtype, int batch, int max_m, int max_n,
@@ -143,7 +145,7 @@ int batched_qr_blocked_max_rows(int dtype);
  * Tiers: the register tier holds min(m, n) <= 64 and max(m, n) <= 128 (F32) / 64 (F64); the shared
  * tier max(m, n) <= 256 and min(m, n) <= 160 (F32, while the matrix and V fit in 220 KiB of shared
  * memory) / 64 (F64); FP32 matrices up to 128 x 128 in the shared tier keep their columns in
- * registers and exchange one column per pair step through shared memory.  BSVD_TIER_AUTO uses the choice
+ * registers and exchange one column per pair slot and step through shared memory.  BSVD_TIER_AUTO uses the choice
  * recorded by bsvd_set_jacobi_choice for the size bin, else the register tier when it fits, else
  * the shared tier; larger shapes give BSVD_ERR_UNSUPPORTED.
  */
@@ -166,7 +168,9 @@ int bsvd_jacobi_variants(int dtype, int max_m, int max_n, int tier);
  * bsvd_jacobi_variant_desc -- describe the k-th (k >= 1) register-tier variant that fits a batch
  * bounded by max_m x max_n (the variant BSVD_TIER_REGISTER | (k << 8) launches).  desc (HOST, 9
  * ints, caller-owned) receives {column-pair slots, row parts, rows of A per lane, rows of V per
- * lane, resident CTAs per SM, scaled rotations (0/1), QR preconditioning (0/1), FP64 rotation
+ * lane, resident CTAs per SM (a request: a batch of more than a few matrices per SM may run the same
+ * arithmetic with the matrix and V in separate warps, 64 x 64 ones six to an SM whatever the figure,
+ * with the same results), scaled rotations (0/1), QR preconditioning (0/1), FP64 rotation
  * parameters (0/1), carried column norms (0/1)}.  QR preconditioning (square bounds only) factors A = Q R and runs the sweeps
  * on R^T (the project's addition; the paper runs them on A).  FP64 rotation parameters (FP32 data
  * only) compute zeta, t, c, s and the rotation test in FP64 from the FP32 Gram sums; carried
