@@ -88,6 +88,9 @@ TRAFFIC = {
     # qr_warp_kernel<float, 128, 1>, 10 000 128x32 matrices: 164.79 MB read + 146.25 MB written, per
     # 20 000-matrix launch (re-captured after the CTA QR kernel's load phase changed in the same file)
     "qr:228caeb56544bd00": 2 * (164.788992e6 + 146.252800e6),
+    # jacobi_wv_kernel<1, 6, true, false, true>, 10 000 64x64 matrices with U and V: 166.25 MB read + 278.54 MB
+    # written, per 20 000-matrix launch
+    "jacobi_wv:e2fef7f32edd7386": 2 * (166.245376e6 + 278.542592e6),
 }
 
 
@@ -236,6 +239,19 @@ def tier_precond(bs, code, m, n, tier):
     return bool(bs.jacobi_variant_desc(code, m, n, k)["qr_precond"])
 
 
+def jacobi_kernel(bs, code, m, n, tier):
+    """The kernel a large batch of the encoded tier launches (csrc/jacobi_reg.cu's and jacobi_smem.cu's rules)."""
+    f32 = code == bs.F32
+    if (tier & 0xff) != bs.TIER_REGISTER:
+        if f32 and max(m, n) <= 128 and min(m, n) > 0:
+            return "jacobi_rx_kernel" if min(m, n) > 16 else "jacobi_rx8_kernel"
+        return "jacobi_smem_kernel"
+    d = bs.jacobi_variant_desc(code, m, n, tier >> 8 or 1)
+    # 32 slots of scaled rotations on parts of 32 rows: the form with W and V in separate warps
+    wv = f32 and d["slots"] == 32 and d["rows_a"] == 32 and d["scaled"]
+    return "jacobi_wv_kernel" if wv else "jacobi_reg_kernel"
+
+
 def max_over_ranks(x, world, dev):
     if world == 1:
         return x
@@ -349,10 +365,10 @@ class SvdQr64:
         fl = jacobi_flops(64, 64, info_h, rots_h, pre)
         achieved = fl / (kernel_ms * 1e-3) / 1e12
         tier = int(self.tuned["tier"])
-        reg = (tier & 0xff) == bs.TIER_REGISTER
-        # (32 slots of scaled rotations: the form with W and V in separate warps)
-        kname = ("jacobi_wv_kernel" if reg else "jacobi_smem_kernel") + f" (tier {tier:#x})"
-        traffic = TRAFFIC.get("jacobi_wv:" + kernel_digest("jacobi_wv.cu")) if reg else None
+        kernel = jacobi_kernel(bs, bs.F32, 64, 64, tier)
+        kname = f"{kernel} (tier {tier:#x})"
+        traffic = (TRAFFIC.get("jacobi_wv:" + kernel_digest("jacobi_wv.cu"))
+                   if pre and kernel == "jacobi_wv_kernel" else None)
         if traffic is not None:
             traffic *= self.nb / 20000  # per launch: scales with the matrix count
         roof = {"kernel": kname, "bound": "alu", "achieved": achieved, "peak": PEAKS["fp32"]["tflops"], "unit": "TFLOP/s",

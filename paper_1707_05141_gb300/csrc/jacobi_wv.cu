@@ -17,11 +17,13 @@
 //            step is two FMAs per pair and row and no exchange: the swap of positions is a renaming of
 //            registers.  The steps' multipliers arrive in a ring in shared memory, broadcast to all
 //            lanes; the V warp runs up to kRing double steps behind the W warps.
-// Why: with W and V in the same lanes (jacobi_reg.cu) a step of a 64 x 64 matrix is 1390 warp
-// instructions, of which 366 are FP32 FMAs; the rest is the exchange of W and V (a shuffle per element,
-// two selects per element on odd steps, moves), parameters computed by both row parts, and spills.
-// Here it is 550, and the step's dependent chain bounds it (one W warp alone: about 1170 cycles a step,
-// 480 of them exchange, 400 parameters, 260 dot products; 12 warps in 168 registers each on an SM).
+// Why: with W and V in the same lanes (jacobi_reg.cu) a preconditioned 64 x 64 matrix takes 759 k warp
+// instructions (1400 a step, of which 366 are FP32 FMAs); the rest is the exchange of W and V (a shuffle
+// per element, two selects per element on odd steps, moves), parameters computed by both row parts, and
+// spills.  Here it takes 357 k (660 a step), and the step's dependent chain of exchange, parameters and dot
+// products bounds it: 1550 cycles a step for a matrix alone; with 12 warps in 168 registers each on an SM
+// 41 % of the issue slots and 32 % of the FMA pipe are busy, and barrier waits (the V warps', for the
+// ring) and fixed latencies lead the stalls.
 // Measured (GB300, before -> after): 20 000 preconditioned 64 x 64 matrices 18.6 -> 13.8 ms; 500 of
 // 512 x 512 by the block tier, whose inner SVDs these are, 230 -> 212 ms; a depth-12 basis tree (128-row
 // form) 16.0 -> 12.4 ms.
