@@ -254,7 +254,8 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(int batch, const float* f
 #pragma unroll
         for (int j = 0; j < 4; ++j) g2[i][j] = 0.f;
     }
-    for (int t0 = blockIdx.x * kTile; t0 < batch; t0 += gridDim.x * kTile) {
+    // (64-bit: the last stride past a batch near 2^31 does not wrap)
+    for (long long t0 = (long long)blockIdx.x * kTile; t0 < batch; t0 += (long long)gridDim.x * kTile) {
         __syncthreads();  // P is there; the previous tile's arrays are free
         for (int e = tid; e < kTile * kF; e += 256) {
             const int s = e / kF, i = e - s * kF;
@@ -468,7 +469,7 @@ int bsvd_mlp_grad(int batch, const float* d_features, const float* d_target, con
             return BSVD_ERR_CUDA;
         // a tile per CTA while they fit the GPU once, then tiles in turn: the additions to global memory
         // are one set per CTA
-        const int tiles = (batch + kTile - 1) / kTile;
+        const int tiles = (batch - 1) / kTile + 1;
         const int grid = persistent_grid(mlp_grad_kernel, 256, kGradSmem, tiles);
         mlp_grad_kernel<<<grid, 256, kGradSmem, st>>>(batch, d_features, d_target, d_params, d_grad, d_loss);
     }
