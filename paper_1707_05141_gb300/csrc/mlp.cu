@@ -232,7 +232,7 @@ constexpr int kTile = 32;             // samples per tile
 constexpr int kLdS = kTile + 4;       // row stride of the activation arrays (unit-major)
 constexpr size_t kGradSmem = sizeof(float) * (((kParams + 3) & ~3) + 3 * kH * kLdS + kTile * (kF + 1) + kTile);
 
-__global__ void __launch_bounds__(256) mlp_grad_kernel(int batch, const float* feat, const float* target,
+__global__ void __launch_bounds__(256, 2) mlp_grad_kernel(int batch, const float* feat, const float* target,
                                                        const float* params, float* grad, float* loss)
 {
     extern __shared__ __align__(16) float sm[];
@@ -243,7 +243,15 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(int batch, const float* f
     float* xs = d2 + kH * kLdS;                     // xs[sample][feature]
     float* dys = xs + kTile * (kF + 1);             // dL/dy
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < kParams; i += 256) P[i] = params[i];
+    // An infinity or a NaN (in a feature, a parameter, or by overflow) must not reach the gradients of units whose
+    // derivative is 0: one bad sample would spoil a batch whose loss it leaves finite.  z is NaN where one occurs,
+    // and such a tile's sums leave out zero derivatives.
+    float z = 0.f;
+    for (int i = tid; i < kParams; i += 256) {
+        P[i] = params[i];
+        z = fmaf(P[i], 0.f, z);
+    }
+    const bool odd_params = __syncthreads_or(z != z);
     const int u0 = warp * 8;                        // this warp's units
     const int o0 = (tid >> 4) * 4, i0 = (tid & 15) * 4;   // this thread's block of dW2
     const int w1o = tid >> 2, w1i = (tid & 3) * 4;  // ... of dW1
@@ -263,8 +271,12 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(int batch, const float* f
         }
         __syncthreads();
         float x[kF], acc[8];
+        z = 0.f;
 #pragma unroll
-        for (int i = 0; i < kF; ++i) x[i] = xs[lane * (kF + 1) + i];
+        for (int i = 0; i < kF; ++i) {
+            x[i] = xs[lane * (kF + 1) + i];
+            z = fmaf(x[i], 0.f, z);
+        }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             acc[u] = P[oB1 + u0 + u];
@@ -277,8 +289,10 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(int batch, const float* f
                 acc[u] = fmaf(w.w, x[i + 3], acc[u]);
             }
             h1[(u0 + u) * kLdS + lane] = acc[u] > 0.f ? acc[u] : 0.f;
+            z = fmaf(acc[u], 0.f, z);
         }
-        __syncthreads();
+        const bool odd = __syncthreads_or(z != z) || odd_params;
+        const bool live = t0 + lane < batch;
 #pragma unroll
         for (int u = 0; u < 8; ++u) acc[u] = P[oB2 + u0 + u];
 #pragma unroll 4
@@ -305,7 +319,6 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(int batch, const float* f
             float y = P[oB3];
 #pragma unroll 16
             for (int i = 0; i < kH; ++i) y = fmaf(P[oW3 + i], h2[i * kLdS + lane], y);
-            const bool live = t0 + lane < batch;
             const float r = live ? y - target[t0 + lane] : 0.f;
             const float dy = r / batch;
             dys[lane] = dy;
@@ -315,55 +328,78 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(int batch, const float* f
         __syncthreads();
         const float dy = dys[lane];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) d2[(u0 + u) * kLdS + lane] = acc[u] > 0.f ? dy * P[oW3 + u0 + u] : 0.f;
+        for (int u = 0; u < 8; ++u) d2[(u0 + u) * kLdS + lane] = acc[u] > 0.f && live ? dy * P[oW3 + u0 + u] : 0.f;
+        const int ns = odd && batch - t0 < kTile ? (int)(batch - t0) : kTile;
         if (tid < kH)
-            for (int s = 0; s < kTile; ++s) gw3 = fmaf(dys[s], h2[tid * kLdS + s], gw3);
+            for (int s = 0; s < ns; ++s) gw3 = fmaf(dys[s], h2[tid * kLdS + s], gw3);
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < 8; ++u) acc[u] = 0.f;
+        if (odd) {
+            for (int o = 0; o < kH; ++o) {
+                const float d = d2[o * kLdS + lane];
+                if (d == 0.f) continue;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) acc[u] = fmaf(P[oW2 + o * kH + u0 + u], d, acc[u]);
+            }
+        } else {
 #pragma unroll 8
-        for (int o = 0; o < kH; ++o) {
-            const float d = d2[o * kLdS + lane];
-            const float4 w0 = *reinterpret_cast<const float4*>(P + oW2 + o * kH + u0);
-            const float4 w1 = *reinterpret_cast<const float4*>(P + oW2 + o * kH + u0 + 4);
-            acc[0] = fmaf(w0.x, d, acc[0]);
-            acc[1] = fmaf(w0.y, d, acc[1]);
-            acc[2] = fmaf(w0.z, d, acc[2]);
-            acc[3] = fmaf(w0.w, d, acc[3]);
-            acc[4] = fmaf(w1.x, d, acc[4]);
-            acc[5] = fmaf(w1.y, d, acc[5]);
-            acc[6] = fmaf(w1.z, d, acc[6]);
-            acc[7] = fmaf(w1.w, d, acc[7]);
+            for (int o = 0; o < kH; ++o) {
+                const float d = d2[o * kLdS + lane];
+                const float4 w0 = *reinterpret_cast<const float4*>(P + oW2 + o * kH + u0);
+                const float4 w1 = *reinterpret_cast<const float4*>(P + oW2 + o * kH + u0 + 4);
+                acc[0] = fmaf(w0.x, d, acc[0]);
+                acc[1] = fmaf(w0.y, d, acc[1]);
+                acc[2] = fmaf(w0.z, d, acc[2]);
+                acc[3] = fmaf(w0.w, d, acc[3]);
+                acc[4] = fmaf(w1.x, d, acc[4]);
+                acc[5] = fmaf(w1.y, d, acc[5]);
+                acc[6] = fmaf(w1.z, d, acc[6]);
+                acc[7] = fmaf(w1.w, d, acc[7]);
+            }
         }
         float* d1 = h2;   // (h2 was last read before the barrier above)
 #pragma unroll
         for (int u = 0; u < 8; ++u)
             d1[(u0 + u) * kLdS + lane] = h1[(u0 + u) * kLdS + lane] > 0.f ? acc[u] : 0.f;
         __syncthreads();
-        // sums over the tile's samples, four at a time
-#pragma unroll 2
-        for (int s = 0; s < kTile; s += 4) {
-            float4 a[4], c[4];
+        if (odd) {
+            for (int s = 0; s < kTile; ++s) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                a[k] = *reinterpret_cast<const float4*>(d2 + (o0 + k) * kLdS + s);
-                c[k] = *reinterpret_cast<const float4*>(h1 + (i0 + k) * kLdS + s);
-            }
+                for (int i = 0; i < 4; ++i) {
+                    const float a = d2[(o0 + i) * kLdS + s], d = d1[w1o * kLdS + s];
+                    if (d != 0.f) g1[i] = fmaf(d, xs[s * (kF + 1) + w1i + i], g1[i]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    g2[i][j] = fmaf(a[i].x, c[j].x, g2[i][j]);
-                    g2[i][j] = fmaf(a[i].y, c[j].y, g2[i][j]);
-                    g2[i][j] = fmaf(a[i].z, c[j].z, g2[i][j]);
-                    g2[i][j] = fmaf(a[i].w, c[j].w, g2[i][j]);
+                    for (int j = 0; j < 4; ++j)
+                        if (a != 0.f) g2[i][j] = fmaf(a, h1[(i0 + j) * kLdS + s], g2[i][j]);
                 }
-        }
-#pragma unroll 4
-        for (int s = 0; s < kTile; ++s) {
-            const float d = d1[w1o * kLdS + s];
+            }
+        } else {
+            // sums over the tile's samples, four at a time
+#pragma unroll 2
+            for (int s = 0; s < kTile; s += 4) {
+                float4 a[4], c[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) g1[i] = fmaf(d, xs[s * (kF + 1) + w1i + i], g1[i]);
+                for (int k = 0; k < 4; ++k) {
+                    a[k] = *reinterpret_cast<const float4*>(d2 + (o0 + k) * kLdS + s);
+                    c[k] = *reinterpret_cast<const float4*>(h1 + (i0 + k) * kLdS + s);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        g2[i][j] = fmaf(a[i].x, c[j].x, g2[i][j]);
+                        g2[i][j] = fmaf(a[i].y, c[j].y, g2[i][j]);
+                        g2[i][j] = fmaf(a[i].z, c[j].z, g2[i][j]);
+                        g2[i][j] = fmaf(a[i].w, c[j].w, g2[i][j]);
+                    }
+            }
+#pragma unroll 4
+            for (int s = 0; s < kTile; ++s) {
+                const float d = d1[w1o * kLdS + s];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) g1[i] = fmaf(d, xs[s * (kF + 1) + w1i + i], g1[i]);
+            }
         }
         if (tid < 2 * kH) {
             const float* d = tid < kH ? d1 + tid * kLdS : d2 + (tid - kH) * kLdS;
