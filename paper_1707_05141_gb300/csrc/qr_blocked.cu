@@ -3,17 +3,18 @@
 //
 // Blocked QR (Algorithm 1 in 32-column panels; the larger factorisations of Section 3.2).  The
 // working matrix X (A, or A^T when m < n: mm x nn with mm >= nn) is factored panel by panel:
-//   panel  the (mm - j0) x 32 panel is factored on chip by the Householder kernel's shared-memory
-//          factorisation (unit-norm reflectors v_c with H_c = I - 2 v_c v_c^T stored in place at and
+//   panel  the (mm - j0) x 32 panel is factored on chip (batched_qr_blocked: in registers, qw_panel_kernel;
+//          preconditioning: by the Householder kernel's shared-memory factorisation; unit-norm reflectors v_c with H_c = I - 2 v_c v_c^T stored in place at and
 //          below the diagonal, R above it, R's diagonal aside), and the panel's compact WY factor T
 //          is formed: H_0 ... H_31 = I - V T V^T with T upper triangular, T(c, c) = 2,
 //          T(0:c, c) = -2 T(0:c, 0:c) V(:, 0:c)^T v_c;
 //   update the trailing columns C = X(j0:, j0+32:) <- (I - V T V^T)^T C = C - V T^T (V^T C), in
 //          32-column tiles, rows streamed through shared memory in chunks (any mm).
-// A panel too tall for one CTA's shared memory is factored by a thread-block cluster of up to 8
-// CTAs, each holding a slab of its rows: per column, the CTAs' partial sums of squares, then their
-// partial products with the panel's other columns, are exchanged through distributed shared memory
-// (two cluster barriers), every CTA forming the same reflector from the same sums.
+// A panel too tall for one CTA is factored by a thread-block cluster of up to 8 CTAs, each holding a slab
+// of its rows, every CTA forming the same reflector from the same sums.  Panels in registers exchange the
+// CTAs' partial products of the pivot with all of the panel's columns through distributed shared memory
+// (one cluster barrier per column); panels in shared memory the partial sums of squares, then the
+// partial products with the columns to its right (two).
 // Preconditioned block Jacobi (the QR preconditioning Section 6.3 names as future work; the same
 // effect as the register tier's preconditioning, at the block level).  With X = Q R, the block tier
 // runs on R^T (nn x nn, lower triangular, rows graded like the singular values): R^T = U~ S V~^T
